@@ -48,7 +48,7 @@ struct AdjArgs {
     float2* khm;          // K^H mm
     const float2* diagc;  // conj(K^diag)
     const double* dJ;     // dJ/d(observables), (Tmax + 1) x B x 3, sorted order
-    double* red2;         // Rg x Bp x 4 partial Ebar per stage
+    double* red2;         // row groups (max) x Bp x 4 partial Ebar per stage
     double* gE;           // B x ldE: dJ/dE_j (sorted order)
     int seg0, seglen;
 };
@@ -62,7 +62,6 @@ __device__ double vjp_local(const AdjArgs& a, int k, int b, int slot, float E, f
     constexpr int NB2 = NB * NB;
     const BatchArgs& m = a.b;
     const int64_t Bp = m.Bp;
-    float2 G[NB2], X[NB2], M[NB2];
     // D = dir . d of the k-point, recomputed where it is used from the (L1-resident)
     // dipoles instead of held in registers
     const float2* dxk = m.dx + (int64_t)k * NB2;
@@ -71,167 +70,279 @@ __device__ double vjp_local(const AdjArgs& a, int k, int b, int slot, float E, f
         const float2 d1 = __ldg(dxk + q), d2 = __ldg(dyk + q);
         return make_float2(dr.x * d1.x + dr.y * d2.x, dr.x * d1.y + dr.y * d2.y);
     };
+    const int64_t e0 = (int64_t)k * NB2 * Bp + b, rec = (int64_t)slot * m.N * Bp + e0;
+    float2 G[NB2];
 #pragma unroll
     for (int q = 0; q < NB2; ++q) {
-        const int64_t i = (int64_t)k * NB2 + q;
-        const int64_t e = i * Bp + b;
-        const float2 l = __ldcg(a.lam + e);
-        float2 g = cscale(l, cl);
-        if (cm != 0.f) g = cfma(make_float2(cm, 0.f), __ldcg(a.mu + e), g);
+        float2 g = cscale(__ldcg(a.lam + e0 + q * Bp), cl);
+        if (cm != 0.f) g = cfma(make_float2(cm, 0.f), __ldcg(a.mu + e0 + q * Bp), g);
         G[q] = g;
-        X[q] = __ldcg(a.recX + (int64_t)slot * m.N * Bp + e);
-        const float2 ds = __ldcg(a.recDS + (int64_t)slot * m.N * Bp + e);
-        const float2 D = Dq(q);
-        M[q] = make_float2(ds.x + E * D.x, ds.y + E * D.y);
     }
+    // two passes, so that M and X are not held together (four bands: 32 registers each)
+    {
+        float2 M[NB2];
+#pragma unroll
+        for (int q = 0; q < NB2; ++q) {
+            const float2 ds = __ldcg(a.recDS + rec + q * Bp), D = Dq(q);
+            M[q] = make_float2(ds.x + E * D.x, ds.y + E * D.y);
+        }
+#pragma unroll
+        for (int n = 0; n < NB; ++n)
+#pragma unroll
+            for (int mm = 0; mm < NB; ++mm) {
+                const int q = n * NB + mm;
+                // (A^+ g - g A^+)_nm = (eps_n - eps_m) g_nm + sum_l (conj(M_ln) g_lm - g_nl conj(M_ml))
+                float2 t1 = gap_times(m.gap[(int64_t)k * NB2 + q], G[q]);
+#pragma unroll
+                for (int l = 0; l < NB; ++l) {
+                    t1 = cadd(t1, cmul(cconj(M[l * NB + n]), G[l * NB + mm]));
+                    t1 = csub(t1, cmul(G[n * NB + l], cconj(M[mm * NB + l])));
+                }
+                a.c1[e0 + q * Bp] = mul_i(t1);
+            }
+    }
+    float2 X[NB2];
+#pragma unroll
+    for (int q = 0; q < NB2; ++q) X[q] = __ldcg(a.recX + rec + q * Bp);
     double ebar = 0.0;
 #pragma unroll
     for (int n = 0; n < NB; ++n)
 #pragma unroll
         for (int mm = 0; mm < NB; ++mm) {
             const int q = n * NB + mm;
-            const int64_t i = (int64_t)k * NB2 + q;
-            // (A^+ g - g A^+)_nm = (eps_n - eps_m) g_nm + sum_l (conj(M_ln) g_lm - g_nl conj(M_ml))
-            float2 t1 = gap_times(m.gap[i], G[q]);
             // (g rho^+ - rho^+ g)_nm = g_nm (f_m - f_n) + sum_l (g_nl conj(X_ml) - conj(X_ln) g_lm)
             float2 t2 = cscale(G[q], m.occ[mm] - m.occ[n]);
             // [D, rho]_nm = D_nm (f_m - f_n) + sum_l (D_nl X_lm - X_nl D_lm)
             float2 t3 = cscale(Dq(q), m.occ[mm] - m.occ[n]);
 #pragma unroll
             for (int l = 0; l < NB; ++l) {
-                t1 = cadd(t1, cmul(cconj(M[l * NB + n]), G[l * NB + mm]));
-                t1 = csub(t1, cmul(G[n * NB + l], cconj(M[mm * NB + l])));
                 t2 = cadd(t2, cmul(G[n * NB + l], cconj(X[mm * NB + l])));
                 t2 = csub(t2, cmul(cconj(X[l * NB + n]), G[l * NB + mm]));
                 t3 = cadd(t3, cmul(Dq(n * NB + l), X[l * NB + mm]));
                 t3 = csub(t3, cmul(X[n * NB + l], Dq(l * NB + mm)));
             }
-            const int64_t e = i * Bp + b;
-            a.c1[e] = mul_i(t1);
-            a.mm[e] = mul_i(t2);
+            a.mm[e0 + q * Bp] = mul_i(t2);
             // Re conj(g) (-i t3) = Re(g) Im(t3) - Im(g) Re(t3)
             ebar += (double)G[q].x * (double)t3.y - (double)G[q].y * (double)t3.x;
         }
     return ebar;
 }
 
+// dynamic shared memory of the adjoint kernel
+struct AdjShared {
+    BatchShared bs;
+    AdjArgs a;
+};
+
+__device__ __forceinline__ AdjShared& adj_shared() { return *reinterpret_cast<AdjShared*>(batch_smem); }
+
+// local part of stage s of step bs.n of the segment (own rows, own trajectories): c1, mm and
+// the Ebar partial of every trajectory
+template <int NB>
+__device__ __forceinline__ void phase_local(int nl, int s) {
+    AdjShared& as = adj_shared();
+    const AdjArgs& a = as.a;
+    BatchShared& bs = as.bs;
+    const BatchArgs& m = bs.a;
+    const StepShared& sh = bs.s;
+    const int tid = threadIdx.x;
+    const float h = *(const volatile float*)&m.dt;  // read here: no loop invariant lives across the calls
+    const int eoff = s == 0 ? 0 : (s == 3 ? 2 : 1);
+    {
+        const int bl = tid % kTileB, kg = tid / kTileB;
+        const int ka = sh.ka, kb = sh.kb;
+        // coefficients of lam and of mu_{s+1} in stage s
+        const float cl = s == 0 || s == 3 ? h / 6.f : h / 3.f;
+        const float cm = s == 3 ? 0.f : (s == 2 ? h : 0.5f * h);
+        double eb = 0.0;
+        if (bl < sh.nb) {
+            const int b = sh.b0 + bl;
+            const float E = (float)m.Etab[(int64_t)b * m.ldE + 2 * (a.seg0 + nl) + eoff];
+            const float2 dr = m.dir[b];
+            for (int k = ka + kg; k < kb; k += kBThreads / kTileB)
+                eb += vjp_local<NB>(a, k, b, nl * 4 + s, E, dr, cl, cm);
+        }
+        bs.obs[kg * kTileB + bl] = eb;
+    }
+    __syncthreads();
+    for (int bl = tid; bl < sh.nb; bl += kBThreads) {
+        double eb = 0.0;
+        for (int kg = 0; kg < kBThreads / kTileB; ++kg) eb += bs.obs[kg * kTileB + bl];
+        a.red2[((int64_t)sh.rg * m.Bp + sh.b0 + bl) * 4 + s] = eb;
+    }
+}
+
+// the four products of the K^H application (calls: they need the registers)
+__device__ __noinline__ void phase_uhm() {
+    AdjShared& as = adj_shared();
+    BatchShared& bs = as.bs;
+    const float2* mm = as.a.mm;
+    const BatchArgs& m = bs.a;
+    const StepShared& sh = bs.s;
+    const int NB2 = m.Nb * m.Nb;
+    const int64_t ra = (int64_t)sh.ka * NB2;
+    if (sh.nb > 0)
+        block_gemm<true>(m.U + ra * m.ldu, m.ldu, m.r, sh.nrows, mm + ra * m.Bp + sh.b0, m.Bp, sh.nb,
+                         m.P + (int64_t)blockIdx.x * m.r * kTileB, kTileB, false, nullptr, nullptr);
+}
+
+__device__ __noinline__ void phase_sy_adj() {
+    AdjShared& as = adj_shared();
+    BatchShared& bs = as.bs;
+    const BatchArgs& m = bs.a;
+    const StepShared& sh = bs.s;
+    if (sh.nb > 0) {
+        const int Rg = sh.Rg;
+        reduce_partials(m.P + (int64_t)sh.tg * Rg * m.r * kTileB, (int64_t)m.r * kTileB, sh.jr0, sh.jr1,
+                        sh.nb, m.S, m.Y + sh.b0, m.Bp,
+                        [&](int, int& g0, int& g1) {
+                            g0 = 0;
+                            g1 = Rg - 1;
+                        },
+                        reinterpret_cast<float2*>(bs.obs));
+    }
+}
+
+template <int NB>
+__device__ __noinline__ void phase_vy() {
+    AdjShared& as = adj_shared();
+    BatchShared& bs = as.bs;
+    const float2 *mm = as.a.mm, *diagc = as.a.diagc;
+    float2* khm = as.a.khm;
+    const BatchArgs& m = bs.a;
+    const StepShared& sh = bs.s;
+    constexpr int NB2 = NB * NB;
+    const int64_t ra = (int64_t)sh.ka * NB2, x0 = ra * m.Bp + sh.b0;
+    if (sh.nb > 0)
+        block_gemm<false>(m.V + ra * m.ldu, m.ldu, sh.nrows, m.r, m.Y + sh.b0, m.Bp, sh.nb, khm + x0, m.Bp,
+                          false, m.kblk ? nullptr : diagc + ra, mm + x0);
+    if (m.kblk) {  // K^H: the conjugate-transposed k = k' blocks
+        __syncthreads();
+        if (sh.nb > 0)
+            kblock_term<NB, true>(m.kblk, mm, khm, m.Bp, (int64_t)sh.ka * NB2, sh.nrows, sh.b0, sh.nb);
+    }
+}
+
+template <int NB>
+__device__ __noinline__ void phase_dense_adj() {
+    AdjShared& as = adj_shared();
+    BatchShared& bs = as.bs;
+    const float2* mm = as.a.mm;
+    float2* khm = as.a.khm;
+    const BatchArgs& m = bs.a;
+    const StepShared& sh = bs.s;
+    constexpr int NB2 = NB * NB;
+    const int64_t ra = (int64_t)sh.ka * NB2;
+    if (sh.nb > 0)
+        block_gemm<false>(m.K + ra * m.N, m.N, sh.nrows, (int)m.N, mm + sh.b0, m.Bp, sh.nb,
+                          khm + ra * m.Bp + sh.b0, m.Bp, false, nullptr, nullptr);
+}
+
+// dJ/dE at this stage's sample: sum of the row-group partials, one warp per trajectory, fixed
+// order
+__device__ __noinline__ void phase_gradient() {
+    AdjShared& as = adj_shared();
+    const AdjArgs& a = as.a;
+    const BatchArgs& m = as.bs.a;
+    const StepShared& sh = as.bs.s;
+    const int tid = threadIdx.x, nl = as.bs.n >> 2, s = as.bs.n & 3, eoff = s == 0 ? 0 : (s == 3 ? 2 : 1);
+    for (int b = sh.b0 + (tid >> 5); b < sh.b0 + sh.nb; b += kBThreads / 32) {
+        double eb = 0.0;
+        for (int g2 = tid & 31; g2 < sh.Rg; g2 += 32) eb += __ldcg(a.red2 + ((int64_t)g2 * m.Bp + b) * 4 + s);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) eb += __shfl_xor_sync(0xffffffffu, eb, o);
+        if ((tid & 31) == 0) a.gE[(int64_t)b * m.ldE + 2 * (a.seg0 + nl) + eoff] += eb;
+    }
+}
+
+// mu_s = c1 + K^H mm of this CTA's block and the step's sum; after the step's last stage
+// lam <- lam + sum of the stage VJPs + direct terms of the observables at step n
+template <int NB>
+__device__ __noinline__ void phase_update() {
+    AdjShared& as = adj_shared();
+    constexpr int NB2 = NB * NB;
+    const AdjArgs& a = as.a;
+    const BatchArgs& m = as.bs.a;
+    const StepShared& sh = as.bs.s;
+    const int tid = threadIdx.x, nl = as.bs.n >> 2, s = as.bs.n & 3;
+    const int nb = sh.nb, b0 = sh.b0, nrows = sh.nrows;
+    const int64_t ra = (int64_t)sh.ka * NB2;
+    for (int e = tid; e < nrows * nb; e += kBThreads) {
+        const int64_t off = (ra + e / nb) * m.Bp + b0 + e % nb;
+        const float2 mu = cadd(__ldcg(a.c1 + off), __ldcg(a.khm + off));
+        a.mu[off] = mu;
+        a.musum[off] = s == 3 ? mu : cadd(__ldcg(a.musum + off), mu);
+    }
+    if (s > 0) return;
+    __syncthreads();
+    const double inv = 1.0 / (double)m.Nk;
+    for (int e = tid; e < nrows * nb; e += kBThreads) {
+        const int64_t i = ra + e / nb;
+        const int b = b0 + e % nb;
+        const int64_t off = i * m.Bp + b;
+        const double* dj = a.dJ + ((int64_t)(a.seg0 + nl) * m.B + b) * 3;
+        const float2 d1 = m.dx[i], v1 = m.vx[i];
+        const int q = (int)(i % NB2);
+        const float wP = (float)(dj[0] * inv), wJ = (float)(dj[1] * inv);
+        const float wo = (q / NB == m.c1 && q % NB == m.c1) ? (float)(dj[2] * inv) : 0.f;
+        float2 l = cadd(__ldcg(a.lam + off), __ldcg(a.musum + off));
+        l = make_float2(l.x + wP * d1.x + wJ * v1.x + wo, l.y + wP * d1.y + wJ * v1.y);
+        a.lam[off] = l;
+    }
+}
+
 template <int NB>
 __global__ void __launch_bounds__(kBThreads, 1) adjoint_kernel(AdjArgs a) {
-    extern __shared__ __align__(16) float2 sm[];
-    float2* sA = sm;
-    float2* sB = sA + kChunk * kLdA;
-    double* sred = reinterpret_cast<double*>(sA + kGemmSmem);
-    __shared__ int abort_s;
+    AdjShared& as = adj_shared();
+    BatchShared& bs = as.bs;
+    volatile StepShared& sh = bs.s;
     const BatchArgs& m = a.b;
     const int tid = threadIdx.x;
-    const int rg = blockIdx.x % m.Rg, tg = blockIdx.x / m.Rg;
-    const int ka = (int)((int64_t)rg * m.Nk / m.Rg), kb = (int)((int64_t)(rg + 1) * m.Nk / m.Rg);
     const int NB2 = NB * NB;
-    const int64_t ra = (int64_t)ka * NB2;
-    const int nrows = (kb - ka) * NB2;
-    const int jr0 = (int)((int64_t)rg * m.r / m.Rg), jr1 = (int)((int64_t)(rg + 1) * m.r / m.Rg);
-    const float h = m.dt;
-    const float cls[4] = {h / 6.f, h / 3.f, h / 3.f, h / 6.f};  // coefficient of lam, stage s
-    const float cms[4] = {0.5f * h, 0.5f * h, h, 0.f};          // coefficient of mu_{s+1}
-    if (tid == 0) abort_s = 0;
+    if (tid == 0) {
+        bs.abort_s = 0;
+        bs.gen = 0;
+        sh.Bact = -1;
+        bs.n = 4 * a.seglen - 1;
+    }
+    copy_args(bs.a, m);
+    copy_args(as.a, a);
     __syncthreads();
-    unsigned gen = 0;
-    bool ok = true;
-    int prev_act = -1;
-    for (int nl = a.seglen - 1; nl >= 0 && ok; --nl) {
-        const int n = a.seg0 + nl;
-        const int Bact = m.act[n];
-        int b0, b1;
-        group_range(Bact, m.Tg, tg, b0, b1);
-        const int nb = b1 - b0;
-        if (prev_act >= 0 && Bact != prev_act && !(ok = bgrid_sync(m, gen, &abort_s))) break;
-        prev_act = Bact;
-        for (int s = 3; s >= 0 && ok; --s) {
-            const int eoff = s == 0 ? 0 : (s == 3 ? 2 : 1);
-            // local part (own rows, own trajectories), Ebar partial per trajectory
-            {
-                const int bl = tid % kTileB, kg = tid / kTileB;
-                double eb = 0.0;
-                if (bl < nb) {
-                    const int b = b0 + bl;
-                    const float E = (float)m.Etab[(int64_t)b * m.ldE + 2 * n + eoff];
-                    const float2 dr = m.dir[b];
-                    for (int k = ka + kg; k < kb; k += kBThreads / kTileB)
-                        eb += vjp_local<NB>(a, k, b, nl * 4 + s, E, dr, cls[s], cms[s]);
-                }
-                sred[kg * kTileB + bl] = eb;
+    // stages in reverse; the counter (4 step + stage) is read from shared memory, so that no
+    // register holds it across the calls
+    volatile int& gs = bs.n;
+    while (gs >= 0) {
+        {
+        const int nl = gs >> 2, s = gs & 3;
+        if (s == 3) {
+            if (tid == 0) {
+                bs.prev_act = sh.Bact;
+                set_step(m, m.act[a.seg0 + nl], NB2, sh);
             }
             __syncthreads();
-            for (int bl = tid; bl < nb; bl += kBThreads) {
-                double eb = 0.0;
-                for (int kg = 0; kg < kBThreads / kTileB; ++kg) eb += sred[kg * kTileB + bl];
-                a.red2[((int64_t)rg * m.Bp + b0 + bl) * 4 + s] = eb;
-            }
-            if (m.mode == TDAGW_LOWRANK) {
-                if (nb > 0)
-                    block_gemm<true>(m.U + ra * m.ldu, m.ldu, m.r, nrows, a.mm + ra * m.Bp + b0, m.Bp, nb,
-                                     m.P + (int64_t)rg * m.r * m.Bp + b0, m.Bp, false, nullptr, nullptr, sA, sB);
-                if (!(ok = bgrid_sync(m, gen, &abort_s))) break;
-            } else {
-                if (!(ok = bgrid_sync(m, gen, &abort_s))) break;
-            }
-            // dJ/dE at this stage's sample: sum of the row-group partials
-            if (rg == 0)
-                for (int b = b0 + tid; b < b1; b += kBThreads) {
-                    double eb = 0.0;
-                    for (int g2 = 0; g2 < m.Rg; ++g2) eb += __ldcg(a.red2 + ((int64_t)g2 * m.Bp + b) * 4 + s);
-                    a.gE[(int64_t)b * m.ldE + 2 * n + eoff] += eb;
-                }
-            if (m.mode == TDAGW_LOWRANK) {
-                for (int e = tid; e < (jr1 - jr0) * nb; e += kBThreads) {
-                    const int j = jr0 + e / nb, b = b0 + e % nb;
-                    float2 sum = make_float2(0.f, 0.f);
-                    for (int g2 = 0; g2 < m.Rg; ++g2)
-                        sum = cadd(sum, __ldcg(m.P + ((int64_t)g2 * m.r + j) * m.Bp + b));
-                    m.Y[(int64_t)j * m.Bp + b] = cscale(sum, m.S[j]);
-                }
-                if (!(ok = bgrid_sync(m, gen, &abort_s))) break;
-                if (nb > 0)
-                    block_gemm<false>(m.V + ra * m.ldu, m.ldu, nrows, m.r, m.Y + b0, m.Bp, nb,
-                                      a.khm + ra * m.Bp + b0, m.Bp, m.kblk == nullptr, a.diagc + ra,
-                                      a.mm + ra * m.Bp + b0, sA, sB);
-                if (m.kblk) {  // K^H: the conjugate-transposed k = k' blocks
-                    __syncthreads();
-                    if (nb > 0) kblock_term<NB, true>(m.kblk, a.mm, a.khm, m.Bp, ra, nrows, b0, nb);
-                }
-            } else {
-                if (nb > 0)
-                    block_gemm<false>(m.K + ra * m.N, m.N, nrows, (int)m.N, a.mm + b0, m.Bp, nb,
-                                      a.khm + ra * m.Bp + b0, m.Bp, false, nullptr, nullptr, sA, sB);
-                // all rows of mm are read before the next stage rewrites them
-                if (!(ok = bgrid_sync(m, gen, &abort_s))) break;
-            }
-            __syncthreads();
-            // mu_s = c1 + K^H mm; accumulate the step's sum
-            for (int e = tid; e < nrows * nb; e += kBThreads) {
-                const int64_t off = (ra + e / nb) * m.Bp + b0 + e % nb;
-                const float2 mu = cadd(__ldcg(a.c1 + off), __ldcg(a.khm + off));
-                a.mu[off] = mu;
-                a.musum[off] = s == 3 ? mu : cadd(__ldcg(a.musum + off), mu);
-            }
-            __syncthreads();
+            const int prev = *(volatile int*)&bs.prev_act;
+            if (prev >= 0 && sh.Bact != prev && !bgrid_sync(m, bs)) return;
         }
-        if (!ok) break;
-        // lam <- lam + sum of stage VJPs + direct terms of the observables at step n
-        const double inv = 1.0 / (double)m.Nk;
-        for (int e = tid; e < nrows * nb; e += kBThreads) {
-            const int64_t i = ra + e / nb;
-            const int b = b0 + e % nb;
-            const int64_t off = i * m.Bp + b;
-            const double* dj = a.dJ + ((int64_t)n * m.B + b) * 3;
-            const float2 d1 = m.dx[i], v1 = m.vx[i];
-            const int q = (int)(i % NB2);
-            const float wP = (float)(dj[0] * inv), wJ = (float)(dj[1] * inv);
-            const float wo = (q / NB == m.c1 && q % NB == m.c1) ? (float)(dj[2] * inv) : 0.f;
-            float2 l = cadd(__ldcg(a.lam + off), __ldcg(a.musum + off));
-            l = make_float2(l.x + wP * d1.x + wJ * v1.x + wo, l.y + wP * d1.y + wJ * v1.y);
-            a.lam[off] = l;
+        phase_local<NB>(nl, s);
         }
+        if (m.mode == TDAGW_LOWRANK) {
+            phase_uhm();
+            if (!bgrid_sync(m, bs)) return;
+            if (sh.rg == 0) phase_gradient();
+            phase_sy_adj();
+            if (!bgrid_sync(m, bs)) return;
+            phase_vy<NB>();
+        } else {
+            if (!bgrid_sync(m, bs)) return;
+            if (sh.rg == 0) phase_gradient();
+            phase_dense_adj<NB>();
+            // all rows of mm are read before the next stage rewrites them
+            if (!bgrid_sync(m, bs)) return;
+        }
+        __syncthreads();
+        phase_update<NB>();
+        __syncthreads();
+        if (tid == 0) gs = gs - 1;
         __syncthreads();
     }
 }
@@ -303,7 +414,7 @@ void adjoint_batched(Ctx& c, const double* dJdobs, double* dJdE, double* dJdpara
     TDAGW_CUDA(cudaMemcpyAsync(dT.p, Ts.data(), B * sizeof(int), cudaMemcpyHostToDevice, s));
     gE.ensure((size_t)B * ldE * sizeof(double));
     TDAGW_CUDA(cudaMemsetAsync(gE.p, 0, (size_t)B * ldE * sizeof(double), s));
-    red2.ensure((size_t)st.Rg * Bp * 4 * sizeof(double));
+    red2.ensure((size_t)std::min(st.G, h.Nk) * Bp * 4 * sizeof(double));
     const size_t sb = (size_t)N * Bp * sizeof(float2);
     for (DevBuf* b : {&c.aLam, &c.aMu, &c.aMusum, &c.aC1, &c.aMm, &c.aKhm}) b->ensure(sb);
     const int64_t rec_slots = 4 * (int64_t)C;
@@ -343,12 +454,11 @@ void adjoint_batched(Ctx& c, const double* dJdobs, double* dJdE, double* dJdpara
     aa.dJ = ddj.as<double>();
     aa.red2 = red2.as<double>();
     aa.gE = gE.as<double>();
-    const size_t smem = (size_t)kGemmSmem * sizeof(float2) +
-                        (size_t)(kBThreads / kTileB) * kTileB * 3 * sizeof(double);
+    const size_t smem = kBatchSmem, bsmem = sizeof(AdjShared);
     const void* ffn = st.fwd_fn;
     const void* bfn = h.Nb == 2 ? (const void*)adjoint_kernel<2> : (const void*)adjoint_kernel<4>;
-    TDAGW_CUDA(cudaFuncSetAttribute(bfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const dim3 grid(st.Rg * st.Tg);
+    TDAGW_CUDA(cudaFuncSetAttribute(bfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsmem));
+    const dim3 grid(st.G);
     const int nseg = (Tmax + C - 1) / C;
     for (int sg = nseg - 1; sg >= 0; --sg) {
         const int n0 = sg * C, len = std::min(C, Tmax - n0);
@@ -370,7 +480,7 @@ void adjoint_batched(Ctx& c, const double* dJdobs, double* dJdE, double* dJdpara
         aa.seglen = len;
         TDAGW_CUDA(cudaMemsetAsync(c.sync.p, 0, 4 * sizeof(unsigned), s));
         void* bargs[] = {&aa};
-        TDAGW_CUDA(cudaLaunchCooperativeKernel(bfn, grid, dim3(kBThreads), bargs, smem, s));
+        TDAGW_CUDA(cudaLaunchCooperativeKernel(bfn, grid, dim3(kBThreads), bargs, bsmem, s));
         c.persistent_launched = true;
     }
     std::vector<double> hg((size_t)B * ldE);

@@ -8,7 +8,8 @@
 // Work split: CTA (rg, tg) owns the pair elements of a k-aligned row group rg and the
 // trajectories of group tg; trajectories are sorted by length (longest first), so the
 // active ones at step n are a prefix of length B_act(n) and each group takes an equal
-// share of that prefix -- finished trajectories cost nothing (compaction by sorting).
+// share of that prefix -- finished trajectories cost nothing (compaction by sorting); the
+// numbers of row and trajectory groups follow the active count (step_plan).
 // Per low-rank stage:
 //   A  P[rg] = V[rows(rg)]^H X[rows(rg), tg]        (partial over the row group)
 //   -- grid barrier --
@@ -17,8 +18,8 @@
 //   D  dSigma[rows(rg), tg] = U[rows(rg)] Y[:, tg] + K^diag o X
 //   E  commutator + RK4 for k in rg, trajectories in tg (rows this CTA just computed)
 // Dense stages: grid barrier (X complete), dSigma[rows(rg), tg] = K[rows(rg)] X[:, tg], E.
-// The matrix products are register-tiled (4 x 4 complex outputs per thread) FP32 FMAs
-// through shared memory.  Grid barriers are bounded waits (as in the single-trajectory
+// The matrix products are register-tiled (8 x 4 complex outputs per thread) FP32 FMAs
+// through shared memory (block_gemm).  Grid barriers are bounded waits (as in the single-trajectory
 // persistent kernel); on expiry the kernel sets an error word and returns.
 #include <algorithm>
 #include <cmath>
@@ -100,231 +101,242 @@ __device__ void stage_kb(const BatchArgs& a, int k, int b, int st, float E, floa
         }
 }
 
+// A: partial V^H X over this row group (channel-wise: one product per input pair q, its V
+// segment's rows of this row group with the rows k P + q of X)
+template <int NB, bool CH>
+__device__ __noinline__ void phase_vhx() {
+    BatchShared& bs = batch_shared();
+    const BatchArgs& a = bs.a;
+    const StepShared& sh = bs.s;
+    constexpr int NB2 = NB * NB;
+    if constexpr (!CH) {
+        const int64_t ra = (int64_t)sh.ka * NB2;
+        if (sh.nb > 0)
+            block_gemm<true>(a.V + ra * a.ldu, a.ldu, a.r, sh.nrows, a.X + ra * a.Bp + sh.b0, a.Bp, sh.nb,
+                             a.P + (int64_t)blockIdx.x * a.r * kTileB, kTileB, false, nullptr, nullptr);
+    } else if (sh.nb > 0) {
+        // channel-wise: q-major row shares as in D below (rows q Nk + k' of the
+        // V segments, one or two input pairs per row group); the group writes the
+        // partials of those pairs' columns only
+        for (int q = sh.u0 / a.Nk; q < NB2 && q * a.Nk < sh.u1; ++q) {
+            const int ldv = a.chm->ldv[q];
+            const int k0 = max(sh.u0 - q * a.Nk, 0), k1 = min(sh.u1 - q * a.Nk, a.Nk);
+            if (ldv == 0 || k1 <= k0) continue;
+            block_gemm<true>(a.Vch + a.chm->vbase[q] + (int64_t)k0 * ldv, ldv, ldv, k1 - k0,
+                             a.X + ((int64_t)k0 * NB2 + q) * a.Bp + sh.b0, (int64_t)NB2 * a.Bp, sh.nb,
+                             a.P + ((int64_t)blockIdx.x * a.r + a.chm->sbase[q]) * kTileB, kTileB, false,
+                             nullptr, nullptr);
+        }
+    }
+}
+
+// C: Y[j][b] = S_j sum over row groups, j in this CTA's slice (channel-wise: over the row
+// groups whose share touches the input pair of column j)
+template <int NB, bool CH>
+__device__ __noinline__ void phase_sy() {
+    BatchShared& bs = batch_shared();
+    const BatchArgs& a = bs.a;
+    const StepShared& sh = bs.s;
+    constexpr int NB2 = NB * NB;
+    if (sh.nb > 0) {
+        const int Rg = sh.Rg;
+        auto range = [&](int j, int& g0, int& g1) {
+            g0 = 0;
+            g1 = Rg - 1;
+            if constexpr (CH) {
+                int q = 0;
+                while (q + 1 < NB2 && a.chm->sbase[q + 1] <= j) ++q;
+                const int64_t NR = a.N, RG = Rg, lo = (int64_t)q * a.Nk;
+                g0 = max(0, (int)(((lo + 1) * RG + NR - 1) / NR) - 1);
+                g1 = min(Rg - 1, (int)(((lo + a.Nk) * RG + NR - 1) / NR) - 1);
+            }
+        };
+        // partials of the row groups of this trajectory group
+        reduce_partials(a.P + (int64_t)sh.tg * Rg * a.r * kTileB, (int64_t)a.r * kTileB, sh.jr0, sh.jr1,
+                        sh.nb, a.S, a.Y + sh.b0, a.Bp, range, reinterpret_cast<float2*>(bs.obs));
+    }
+}
+
+template <int NB, bool CH>
+__device__ __noinline__ void phase_uy() {
+    BatchShared& bs = batch_shared();
+    const BatchArgs& a = bs.a;
+    const StepShared& sh = bs.s;
+    constexpr int NB2 = NB * NB;
+    if constexpr (!CH) {
+        // D: dSigma = U Y + K^diag X for this row group (the strict diagonal fused
+        // into the product, or the k = k' blocks added after it)
+        const int64_t ra = (int64_t)sh.ka * NB2, x0 = ra * a.Bp + sh.b0;
+        if (sh.nb > 0)
+            block_gemm<false>(a.U + ra * a.ldu, a.ldu, sh.nrows, a.r, a.Y + sh.b0, a.Bp, sh.nb, a.dS + x0,
+                              a.Bp, false, a.kblk ? nullptr : a.diag + ra, a.X + x0);
+        if (a.kblk) {
+            __syncthreads();  // this CTA's U Y rows are written
+            if (sh.nb > 0)
+                kblock_term<NB, false>(a.kblk, a.X, a.dS, a.Bp, (int64_t)sh.ka * NB2, sh.nrows, sh.b0, sh.nb);
+        }
+    } else {
+        // D (channel-wise) by p-major shares: row group rg takes the rows
+        // [u0, u1) of the order p Nk + k (one or two output pairs), so each pair
+        // is one product over many k-points instead of the group's few: the dense
+        // diagonal channel with x_p over all k, then each off-diagonal channel's
+        // U^pq with its block of S o Y added.  The rows reach their k-point's
+        // owner through global memory across the barrier below.
+        const int64_t ldo = (int64_t)NB2 * a.Bp;
+        if (sh.nb > 0)
+            for (int p = sh.u0 / a.Nk; p < NB2 && p * a.Nk < sh.u1; ++p) {
+                const int k0 = max(sh.u0 - p * a.Nk, 0), k1 = min(sh.u1 - p * a.Nk, a.Nk);
+                if (k1 <= k0) continue;
+                const int ldw = a.chm->ldw[p];
+                const float2* Ub = a.Uch + a.chm->ubase[p] + (int64_t)k0 * ldw;
+                float2* o = a.dS + ((int64_t)k0 * NB2 + p) * a.Bp + sh.b0;
+                block_gemm<false>(Ub + a.chm->nlr[p], ldw, k1 - k0, a.Nk, a.X + (int64_t)p * a.Bp + sh.b0,
+                                  ldo, sh.nb, o, ldo, false, nullptr, nullptr);
+                for (int q = 0; q < NB2; ++q) {
+                    const int z = a.choff[2 * NB2 * NB2 + p * NB2 + q];
+                    if (q == p || z == 0) continue;
+                    const int64_t yrow = a.chm->sbase[q] + a.choff[NB2 * NB2 + q * NB2 + p];
+                    block_gemm<false>(Ub + a.choff[p * NB2 + q], ldw, k1 - k0, z,
+                                      a.Y + yrow * a.Bp + sh.b0, a.Bp, sh.nb, o, ldo, true, nullptr,
+                                      nullptr);
+                }
+            }
+    }
+}
+
+// dense mode: dSigma rows of this row group
+template <int NB>
+__device__ __noinline__ void phase_dense() {
+    BatchShared& bs = batch_shared();
+    const BatchArgs& a = bs.a;
+    const StepShared& sh = bs.s;
+    constexpr int NB2 = NB * NB;
+    const int64_t ra = (int64_t)sh.ka * NB2;
+    if (sh.nb > 0)
+        block_gemm<false>(a.K + ra * a.N, a.N, sh.nrows, (int)a.N, a.X + sh.b0, a.Bp, sh.nb,
+                          a.dS + ra * a.Bp + sh.b0, a.Bp, false, nullptr, nullptr);
+}
+
+// Records, commutator + RK4 stage update and observables partials of this CTA's block (k in
+// [ka, kb), trajectories [b0, b0 + nb)), stage gs of the launch.
+template <int NB>
+__device__ __forceinline__ void epilogue(const BatchArgs& a, BatchShared& bs, int gs) {
+    constexpr int NB2 = NB * NB;
+    volatile StepShared& sh = bs.s;
+    const int tid = threadIdx.x, n = gs >> 2, st = gs & 3;
+    const int nb = sh.nb, b0 = sh.b0, ka = sh.ka, kb = sh.kb;
+    if (a.recX) {
+        // stage input and dSigma of this stage, for the adjoint's backward sweep
+        const int64_t slot = (int64_t)(n * 4 + st) * a.N * a.Bp, ra = (int64_t)ka * NB2;
+        for (int e = threadIdx.x; e < (kb - ka) * NB2 * nb; e += kBThreads) {
+            const int64_t off = (ra + e / nb) * a.Bp + b0 + e % nb;
+            a.recX[slot + off] = __ldcg(a.X + off);
+            a.recDS[slot + off] = __ldcg(a.dS + off);
+        }
+    }
+    // E: commutator + RK4 for (k in [ka, kb), b in [b0, b1))
+    const int eoff = st == 0 ? 0 : (st == 3 ? 2 : 1);
+    {
+        const int bl = tid % kTileB, kg = tid / kTileB;  // 16 k-groups x 32 trajectories
+        ObsDF ob;
+        if (bl < nb) {
+            const int b = b0 + bl;
+            const float E = (float)a.Etab[(int64_t)b * a.ldE + 2 * (a.n0 + n) + eoff];
+            const float2 dr = a.dir[b];
+            for (int k = ka + kg; k < kb; k += kBThreads / kTileB) stage_kb<NB>(a, k, b, st, E, dr, ob);
+        }
+        if (st == 3) {
+            bs.obs[(kg * kTileB + bl) * 3] = ob.p.value();
+            bs.obs[(kg * kTileB + bl) * 3 + 1] = ob.j.value();
+            bs.obs[(kg * kTileB + bl) * 3 + 2] = ob.o.value();
+        }
+    }
+    __syncthreads();
+    if (st == 3)
+        for (int bl = tid; bl < nb; bl += kBThreads) {
+            double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+            for (int kg = 0; kg < kBThreads / kTileB; ++kg) {
+                s0 += bs.obs[(kg * kTileB + bl) * 3];
+                s1 += bs.obs[(kg * kTileB + bl) * 3 + 1];
+                s2 += bs.obs[(kg * kTileB + bl) * 3 + 2];
+            }
+            double* rr = a.red + ((int64_t)sh.rg * a.Bp + b0 + bl) * 3;
+            rr[0] = s0;
+            rr[1] = s1;
+            rr[2] = s2;
+        }
+    __syncthreads();
+}
+
 // CH: the channel-wise mode (a separate instantiation, so the other modes' code is unchanged)
 template <int NB, bool CH>
 __global__ void __launch_bounds__(kBThreads, 1) batched_kernel(BatchArgs a) {
-    extern __shared__ __align__(16) float2 sm[];
-    float2* sA = sm;                       // kChunk x kLdA
-    float2* sB = sA + kChunk * kLdA;       // kChunk x 32
-    double* sred = reinterpret_cast<double*>(sA + kGemmSmem);  // 16 x kTileB x 3
-    __shared__ int abort_s;
+    BatchShared& bs = batch_shared();
+    volatile StepShared& sh = bs.s;
     const int tid = threadIdx.x;
-    const int rg = blockIdx.x % a.Rg, tg = blockIdx.x / a.Rg;
-    const int ka = (int)((int64_t)rg * a.Nk / a.Rg), kb = (int)((int64_t)(rg + 1) * a.Nk / a.Rg);
-    const int NB2 = NB * NB;
-    const int64_t ra = (int64_t)ka * NB2;
-    const int nrows = (kb - ka) * NB2;
-    const int jr0 = (int)((int64_t)rg * a.r / a.Rg), jr1 = (int)((int64_t)(rg + 1) * a.r / a.Rg);
-    if (tid == 0) abort_s = 0;
+    constexpr int NB2 = NB * NB;
+    if (tid == 0) {
+        bs.abort_s = 0;
+        bs.gen = 0;
+        sh.Bact = -1;
+    }
+    copy_args(bs.a, a);
     __syncthreads();
-    unsigned gen = 0;
-    bool ok = true;
-    int prev_act = -1;
-    for (int n = 0; n < a.Tmax && ok; ++n) {
-        const int Bact = a.act[a.n0 + n];
-        int b0, b1;
-        group_range(Bact, a.Tg, tg, b0, b1);
-        const int nb = b1 - b0;
-        if (a.ckS && (a.n0 + n) % a.ck_period == 0) {
-            // checkpoint of the compensated state at the start of step n0 + n (own block)
+    // observables of step n - 1's end (row n), from the split of that step
+    auto last_observables = [&](int n) {
+        const StepPlan pp = step_plan(a.act[a.n0 + n - 1], gridDim.x, a.Nk);
+        if (blockIdx.x % pp.Rg == 0 && blockIdx.x / pp.Rg < (unsigned)pp.Tg)
+            reduce_observables_row(a, n, pp, blockIdx.x / pp.Rg);
+    };
+    for (int gs = 0; gs < 4 * a.Tmax; ++gs) {  // one counter for step and stage: it lives across the calls
+        const int n = gs >> 2;
+        const int st = gs & 3;
+        if (st == 0) {
+            // this step's block of the split
+            if (tid == 0) {
+                bs.prev_act = sh.Bact;
+                set_step(a, a.act[a.n0 + n], NB2, sh);
+            }
+            __syncthreads();
+        }
+        // the dense product and the channel-wise row shares read every CTA's rows of X
+        const bool need_x_barrier = (a.mode == TDAGW_FULL || CH) ? !(n == 0 && st == 0)
+                                                                 : (st == 0 && sh.Bact != *(volatile int*)&bs.prev_act && n > 0);
+        if (need_x_barrier && !bgrid_sync(a, bs)) return;
+        if (st == 0 && a.ckS && (a.n0 + n) % a.ck_period == 0) {
+            // checkpoint of the compensated state at the start of step n0 + n (own block,
+            // complete: a barrier precedes every change of the split)
             const int64_t slot = (int64_t)((a.n0 + n) / a.ck_period) * a.N * a.Bp;
+            const int nb = sh.nb, b0 = sh.b0, nrows = sh.nrows;
+            const int64_t ra = (int64_t)sh.ka * NB2;
             for (int e = threadIdx.x; e < nrows * nb; e += kBThreads) {
                 const int64_t off = (ra + e / nb) * a.Bp + b0 + e % nb;
                 a.ckS[slot + off] = __ldcg(a.Ssum + off);
                 a.ckC[slot + off] = __ldcg(a.Ccomp + off);
             }
         }
-        for (int st = 0; st < 4 && ok; ++st) {
-            // the dense product and the channel-wise row shares read every CTA's rows of X
-            const bool need_x_barrier = (a.mode == TDAGW_FULL || CH) ? !(n == 0 && st == 0)
-                                                                     : (st == 0 && Bact != prev_act && n > 0);
-            if (need_x_barrier && !(ok = bgrid_sync(a, gen, &abort_s))) break;
-            if (st == 0 && n > 0 && rg == 0 && a.mode == TDAGW_FULL) {
-                // observables of step n-1 for this group's trajectories at that step
-                int p0, p1;
-                group_range(a.act[a.n0 + n - 1], a.Tg, tg, p0, p1);
-                for (int b = p0 + tid; b < p1; b += kBThreads) {
-                    double s0 = 0, s1 = 0, s2 = 0;
-                    for (int g2 = 0; g2 < a.Rg; ++g2) {
-                        s0 += __ldcg(a.red + ((int64_t)g2 * a.Bp + b) * 3);
-                        s1 += __ldcg(a.red + ((int64_t)g2 * a.Bp + b) * 3 + 1);
-                        s2 += __ldcg(a.red + ((int64_t)g2 * a.Bp + b) * 3 + 2);
-                    }
-                    double* o = a.obs + ((int64_t)n * a.B + b) * 3;
-                    o[0] = s0 / a.Nk;
-                    o[1] = s1 / a.Nk;
-                    o[2] = s2 / a.Nk;
-                }
-            }
-            if (a.mode != TDAGW_FULL) {
-                // A: partial V^H X over this row group (channel-wise: one product per input
-                // pair q, its V segment's rows of this row group with the rows k P + q of X)
-                if constexpr (!CH) {
-                    if (nb > 0)
-                        block_gemm<true>(a.V + ra * a.ldu, a.ldu, a.r, nrows, a.X + ra * a.Bp + b0, a.Bp, nb,
-                                         a.P + (int64_t)rg * a.r * a.Bp + b0, a.Bp, false, nullptr, nullptr,
-                                         sA, sB);
-                } else if (nb > 0) {
-                    // channel-wise: q-major row shares as in D below (rows q Nk + k' of the
-                    // V segments, one or two input pairs per row group); the group writes the
-                    // partials of those pairs' columns only
-                    const int u0 = (int)((int64_t)rg * a.N / a.Rg), u1 = (int)((int64_t)(rg + 1) * a.N / a.Rg);
-                    for (int q = u0 / a.Nk; q < NB2 && q * a.Nk < u1; ++q) {
-                        const int ldv = a.chm->ldv[q];
-                        const int k0 = max(u0 - q * a.Nk, 0), k1 = min(u1 - q * a.Nk, a.Nk);
-                        if (ldv == 0 || k1 <= k0) continue;
-                        block_gemm<true>(a.Vch + a.chm->vbase[q] + (int64_t)k0 * ldv, ldv, ldv, k1 - k0,
-                                         a.X + ((int64_t)k0 * NB2 + q) * a.Bp + b0, (int64_t)NB2 * a.Bp, nb,
-                                         a.P + ((int64_t)rg * a.r + a.chm->sbase[q]) * a.Bp + b0, a.Bp, false,
-                                         nullptr, nullptr, sA, sB);
-                    }
-                }
-                if (!(ok = bgrid_sync(a, gen, &abort_s))) break;
-                if (st == 0 && n > 0 && rg == 0) {
-                    int p0, p1;
-                    group_range(a.act[a.n0 + n - 1], a.Tg, tg, p0, p1);
-                    for (int b = p0 + tid; b < p1; b += kBThreads) {
-                        double s0 = 0, s1 = 0, s2 = 0;
-                        for (int g2 = 0; g2 < a.Rg; ++g2) {
-                            s0 += __ldcg(a.red + ((int64_t)g2 * a.Bp + b) * 3);
-                            s1 += __ldcg(a.red + ((int64_t)g2 * a.Bp + b) * 3 + 1);
-                            s2 += __ldcg(a.red + ((int64_t)g2 * a.Bp + b) * 3 + 2);
-                        }
-                        double* o = a.obs + ((int64_t)n * a.B + b) * 3;
-                        o[0] = s0 / a.Nk;
-                        o[1] = s1 / a.Nk;
-                        o[2] = s2 / a.Nk;
-                    }
-                }
-                // C: Y[j][b] = S_j sum over row groups, j in this CTA's slice (channel-wise:
-                // over the row groups whose share touches the input pair of column j)
-                for (int e = tid; e < (jr1 - jr0) * nb; e += kBThreads) {
-                    const int j = jr0 + e / nb, b = b0 + e % nb;
-                    int g0 = 0, g1 = a.Rg - 1;
-                    if constexpr (CH) {
-                        int q = 0;
-                        while (q + 1 < NB2 && a.chm->sbase[q + 1] <= j) ++q;
-                        const int64_t NR = a.N, RG = a.Rg, lo = (int64_t)q * a.Nk;
-                        g0 = max(0, (int)(((lo + 1) * RG + NR - 1) / NR) - 1);
-                        g1 = min(a.Rg - 1, (int)(((lo + a.Nk) * RG + NR - 1) / NR) - 1);
-                    }
-                    float2 s = make_float2(0.f, 0.f);
-                    for (int g2 = g0; g2 <= g1; ++g2)
-                        s = cadd(s, __ldcg(a.P + ((int64_t)g2 * a.r + j) * a.Bp + b));
-                    a.Y[(int64_t)j * a.Bp + b] = cscale(s, a.S[j]);
-                }
-                if (!(ok = bgrid_sync(a, gen, &abort_s))) break;
-                if constexpr (!CH) {
-                    // D: dSigma = U Y + K^diag X for this row group (the strict diagonal fused
-                    // into the product, or the k = k' blocks added after it)
-                    if (nb > 0)
-                        block_gemm<false>(a.U + ra * a.ldu, a.ldu, nrows, a.r, a.Y + b0, a.Bp, nb,
-                                          a.dS + ra * a.Bp + b0, a.Bp, a.kblk == nullptr, a.diag + ra,
-                                          a.X + ra * a.Bp + b0, sA, sB);
-                    if (a.kblk) {
-                        __syncthreads();  // this CTA's U Y rows are written
-                        if (nb > 0) kblock_term<NB, false>(a.kblk, a.X, a.dS, a.Bp, ra, nrows, b0, nb);
-                    }
-                } else {
-                    // D (channel-wise) by p-major shares: row group rg takes the rows
-                    // [u0, u1) of the order p Nk + k (one or two output pairs), so each pair
-                    // is one product over many k-points instead of the group's few: the dense
-                    // diagonal channel with x_p over all k, then each off-diagonal channel's
-                    // U^pq with its block of S o Y added.  The rows reach their k-point's
-                    // owner through global memory across the barrier below.
-                    const int64_t ldo = (int64_t)NB2 * a.Bp;
-                    const int u0 = (int)((int64_t)rg * a.N / a.Rg), u1 = (int)((int64_t)(rg + 1) * a.N / a.Rg);
-                    if (nb > 0)
-                        for (int p = u0 / a.Nk; p < NB2 && p * a.Nk < u1; ++p) {
-                            const int k0 = max(u0 - p * a.Nk, 0), k1 = min(u1 - p * a.Nk, a.Nk);
-                            if (k1 <= k0) continue;
-                            const int ldw = a.chm->ldw[p], nl = a.chm->nlr[p];
-                            const float2* Ub = a.Uch + a.chm->ubase[p] + (int64_t)k0 * ldw;
-                            float2* o = a.dS + ((int64_t)k0 * NB2 + p) * a.Bp + b0;
-                            block_gemm<false>(Ub + nl, ldw, k1 - k0, a.Nk, a.X + (int64_t)p * a.Bp + b0, ldo, nb, o,
-                                              ldo, false, nullptr, nullptr, sA, sB);
-                            for (int q = 0; q < NB2; ++q) {
-                                const int z = a.choff[2 * NB2 * NB2 + p * NB2 + q];
-                                if (q == p || z == 0) continue;
-                                const int64_t yrow = a.chm->sbase[q] + a.choff[NB2 * NB2 + q * NB2 + p];
-                                block_gemm<false, true>(Ub + a.choff[p * NB2 + q], ldw, k1 - k0, z,
-                                                        a.Y + yrow * a.Bp + b0, a.Bp, nb, o, ldo, false, nullptr,
-                                                        nullptr, sA, sB);
-                            }
-                        }
-                    // every CTA has read all rows of X before any CTA rewrites its rows
-                    if (!(ok = bgrid_sync(a, gen, &abort_s))) break;
-                }
-            } else {
-                if (nb > 0)
-                    block_gemm<false>(a.K + ra * a.N, a.N, nrows, (int)a.N, a.X + b0, a.Bp, nb,
-                                      a.dS + ra * a.Bp + b0, a.Bp, false, nullptr, nullptr, sA, sB);
-                // every CTA has read all rows of X before any CTA rewrites its rows
-                if (!(ok = bgrid_sync(a, gen, &abort_s))) break;
-            }
-            __syncthreads();
-            if (a.recX) {
-                // stage input and dSigma of this stage, for the adjoint's backward sweep
-                const int64_t slot = (int64_t)(n * 4 + st) * a.N * a.Bp;
-                for (int e = threadIdx.x; e < nrows * nb; e += kBThreads) {
-                    const int64_t off = (ra + e / nb) * a.Bp + b0 + e % nb;
-                    a.recX[slot + off] = __ldcg(a.X + off);
-                    a.recDS[slot + off] = __ldcg(a.dS + off);
-                }
-            }
-            // E: commutator + RK4 for (k in [ka, kb), b in [b0, b1))
-            const int eoff = st == 0 ? 0 : (st == 3 ? 2 : 1);
-            {
-                const int bl = tid % kTileB, kg = tid / kTileB;  // 16 k-groups x 32 trajectories
-                ObsDF ob;
-                if (bl < nb) {
-                    const int b = b0 + bl;
-                    const float E = (float)a.Etab[(int64_t)b * a.ldE + 2 * (a.n0 + n) + eoff];
-                    const float2 dr = a.dir[b];
-                    for (int k = ka + kg; k < kb; k += kBThreads / kTileB) stage_kb<NB>(a, k, b, st, E, dr, ob);
-                }
-                if (st == 3) {
-                    sred[(kg * kTileB + bl) * 3] = ob.p.value();
-                    sred[(kg * kTileB + bl) * 3 + 1] = ob.j.value();
-                    sred[(kg * kTileB + bl) * 3 + 2] = ob.o.value();
-                }
-            }
-            __syncthreads();
-            if (st == 3)
-                for (int bl = tid; bl < nb; bl += kBThreads) {
-                    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-                    for (int kg = 0; kg < kBThreads / kTileB; ++kg) {
-                        s0 += sred[(kg * kTileB + bl) * 3];
-                        s1 += sred[(kg * kTileB + bl) * 3 + 1];
-                        s2 += sred[(kg * kTileB + bl) * 3 + 2];
-                    }
-                    double* rr = a.red + ((int64_t)rg * a.Bp + b0 + bl) * 3;
-                    rr[0] = s0;
-                    rr[1] = s1;
-                    rr[2] = s2;
-                }
-            __syncthreads();
+        // observables of step n-1 (written by the CTAs of that step's row group 0)
+        if (st == 0 && n > 0 && a.mode == TDAGW_FULL) last_observables(n);
+        if (a.mode != TDAGW_FULL) {
+            phase_vhx<NB, CH>();
+            if (!bgrid_sync(a, bs)) return;
+            if (st == 0 && n > 0) last_observables(n);
+            phase_sy<NB, CH>();
+            if (!bgrid_sync(a, bs)) return;
+            phase_uy<NB, CH>();
+            // channel-wise: every CTA has read all rows of X (and written its dSigma rows)
+            // before any CTA rewrites its rows
+            if (CH && !bgrid_sync(a, bs)) return;
+        } else {
+            phase_dense<NB>();
+            // every CTA has read all rows of X before any CTA rewrites its rows
+            if (!bgrid_sync(a, bs)) return;
         }
-        prev_act = Bact;
+        __syncthreads();
+        epilogue<NB>(a, bs, gs);
     }
     // observables of the last step
-    if (ok && a.Tmax > 0 && bgrid_sync(a, gen, &abort_s) && rg == 0) {
-        const int n = a.Tmax;
-        int p0, p1;
-        group_range(a.act[a.n0 + n - 1], a.Tg, tg, p0, p1);
-        for (int b = p0 + tid; b < p1; b += kBThreads) {
-            double s0 = 0, s1 = 0, s2 = 0;
-            for (int g2 = 0; g2 < a.Rg; ++g2) {
-                s0 += __ldcg(a.red + ((int64_t)g2 * a.Bp + b) * 3);
-                s1 += __ldcg(a.red + ((int64_t)g2 * a.Bp + b) * 3 + 1);
-                s2 += __ldcg(a.red + ((int64_t)g2 * a.Bp + b) * 3 + 2);
-            }
-            double* o = a.obs + ((int64_t)n * a.B + b) * 3;
-            o[0] = s0 / a.Nk;
-            o[1] = s1 / a.Nk;
-            o[2] = s2 / a.Nk;
-        }
-    }
+    if (a.Tmax > 0 && bgrid_sync(a, bs)) last_observables(a.Tmax);
 }
 
 }  // namespace
@@ -354,15 +366,11 @@ __global__ void unpermute_kernel(const double* __restrict__ src, double* __restr
     for (int q = 0; q < 3; ++q) dst[(n * B + perm[b]) * 3 + q] = src[e * 3 + q];
 }
 
-struct BatchPlan {
-    int Rg = 0, Tg = 0;
-};
-
 }  // namespace
 
 // Host driver of the batched path (complex64 contexts).  Trajectories are sorted by length
-// (longest first); the block shape (row groups x trajectory groups) is picked by timing a
-// few steps of each candidate (cached per context for this mode, batch size and rank).
+// (longest first); the split into row and trajectory groups follows the active count step by
+// step (step_plan), so no call has to be tuned first.
 BatchSetup prepare_batch(Ctx& c, const tdagw_field* fields, int B, const int* steps, double dt) {
     const HostModel& h = c.hm;
     cudaStream_t s = c.stream;
@@ -507,6 +515,16 @@ void finish_batch(Ctx& c, const BatchSetup& bs, int B) {
     c.obs_B = B;
 }
 
+// Partial products, S o Y and observables partials of a launch over G CTAs.
+static void batch_buffers(Ctx& c, BatchArgs& a, int G, int r, int Bp) {
+    c.bP.ensure((size_t)G * std::max(r, 1) * kTileB * sizeof(float2));
+    c.bY.ensure((size_t)std::max(r, 1) * Bp * sizeof(float2));
+    c.bred.ensure((size_t)std::min(G, c.hm.Nk) * Bp * 3 * sizeof(double));
+    a.P = c.bP.as<float2>();
+    a.Y = c.bY.as<float2>();
+    a.red = c.bred.as<double>();
+}
+
 void propagate_batched(Ctx& c, const tdagw_field* fields, int B, const int* steps, double dt,
                        int mode, int flags) {
     TDAGW_REQUIRE(c.dtype == TDAGW_C64, TDAGW_ERR_UNSUPPORTED, "batched propagation needs a complex64 context");
@@ -528,8 +546,7 @@ void propagate_batched(Ctx& c, const tdagw_field* fields, int B, const int* step
     int dev = 0, nsm = 0;
     TDAGW_CUDA(cudaGetDevice(&dev));
     TDAGW_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    const size_t smem = (size_t)kGemmSmem * sizeof(float2) +
-                        (size_t)(kBThreads / kTileB) * kTileB * 3 * sizeof(double);
+    const size_t smem = kBatchSmem;
     const bool ch = mode == TDAGW_CHANNEL;
     const void* fn = h.Nb == 2 ? (ch ? (const void*)batched_kernel<2, true> : (const void*)batched_kernel<2, false>)
                                : (ch ? (const void*)batched_kernel<4, true> : (const void*)batched_kernel<4, false>);
@@ -537,7 +554,6 @@ void propagate_batched(Ctx& c, const tdagw_field* fields, int B, const int* step
     int per_sm = 0;
     TDAGW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBThreads, smem));
     TDAGW_REQUIRE(per_sm >= 1, TDAGW_ERR_UNSUPPORTED, "batched kernel does not fit on this device");
-    const int max_ctas = nsm * per_sm;
 
     BatchArgs a{};
     a.U = c.U.as<float2>();
@@ -595,74 +611,10 @@ void propagate_batched(Ctx& c, const tdagw_field* fields, int B, const int* step
     a.bar = reinterpret_cast<unsigned long long*>(c.sync.p);
     a.err = reinterpret_cast<int*>(c.sync.as<unsigned>() + 2);
 
-    auto run = [&](const BatchPlan& pl, int T) {
-        a.Rg = pl.Rg;
-        a.Tg = pl.Tg;
-        a.Tmax = T;
-        c.bP.ensure((size_t)std::max(1, pl.Rg * std::max(r, 1)) * Bp * sizeof(float2));
-        c.bY.ensure((size_t)std::max(r, 1) * Bp * sizeof(float2));
-        c.bred.ensure((size_t)pl.Rg * Bp * 3 * sizeof(double));
-        a.P = c.bP.as<float2>();
-        a.Y = c.bY.as<float2>();
-        a.red = c.bred.as<double>();
-        launch_batched(c, fn, dim3(pl.Rg * pl.Tg), dim3(kBThreads), smem, &a, sizeof(a),
-                       {{c.bX.p, sbytes}, {c.bS.p, sbytes}, {c.bC.p, sbytes}, {c.sync.p, 4 * sizeof(unsigned)}},
-                       !(flags & TDAGW_FLAG_NO_GRAPH) && !a.extra_arrivals);
-        c.persistent_launched = true;
-    };
-
-    const uint64_t key = ((uint64_t)mode << 56) | ((uint64_t)B << 32) | (uint64_t)(uint32_t)r;
-    const int tg_min = (B + kTileB - 1) / kTileB;  // at most kTileB trajectories per block
-    BatchPlan plan;
-    const bool test_timeout = (flags & TDAGW_FLAG_TEST_TIMEOUT) != 0;
-    auto it = c.batch_plans.find(key);
-    if (test_timeout) {
-        // timeout test: the first candidate untuned; the launch below waits for an arrival
-        // that never comes
-        plan = {std::min(h.Nk, max_ctas / tg_min), tg_min};
-    } else if (it != c.batch_plans.end()) {
-        plan.Rg = it->second.first;
-        plan.Tg = it->second.second;
-        TDAGW_REQUIRE(plan.Tg >= tg_min && plan.Rg >= 1 && plan.Rg <= h.Nk && plan.Rg * plan.Tg <= max_ctas,
-                      TDAGW_ERR_CUDA, "cached batched launch plan does not fit the call");
-    } else {
-        // candidates: at most 32 trajectories per block (the register tile), CTAs <= SMs
-        std::vector<BatchPlan> cands;
-        for (int tg = tg_min; tg <= std::min(B, 8 * tg_min); tg *= 2) {
-            const int rg = std::min(h.Nk, max_ctas / tg);
-            if (rg >= 1) cands.push_back({rg, tg});
-        }
-        TDAGW_REQUIRE(!cands.empty(), TDAGW_ERR_UNSUPPORTED, "too many trajectories for one launch");
-        if (cands.size() == 1 || Tmax < 8) {
-            plan = cands[0];
-        } else {
-            cudaEvent_t e0, e1;
-            TDAGW_CUDA(cudaEventCreate(&e0));
-            TDAGW_CUDA(cudaEventCreate(&e1));
-            float best = 1e30f;
-            for (const BatchPlan& pl : cands) {
-                run(pl, 2);  // warm
-                TDAGW_CUDA(cudaEventRecord(e0, s));
-                run(pl, 6);
-                TDAGW_CUDA(cudaEventRecord(e1, s));
-                TDAGW_CUDA(cudaEventSynchronize(e1));
-                float ms = 0.f;
-                TDAGW_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-                if (ms < best) {
-                    best = ms;
-                    plan = pl;
-                }
-            }
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-            int err = 0;
-            TDAGW_CUDA(cudaMemcpy(&err, c.sync.as<unsigned>() + 2, sizeof(int), cudaMemcpyDeviceToHost));
-            TDAGW_REQUIRE(!err, TDAGW_ERR_TIMEOUT, "a bounded wait gave up while tuning the batched kernel");
-            // the tuning runs overwrote the observables: restore the first row
-            reset_batch_observables(c, bs, B);
-        }
-        c.batch_plans[key] = {plan.Rg, plan.Tg};
-    }
+    const int G = nsm;  // one CTA per SM (the staging memory fills it)
+    TDAGW_REQUIRE((B + kTileB - 1) / kTileB <= G, TDAGW_ERR_UNSUPPORTED, "too many trajectories for one launch");
+    batch_buffers(c, a, G, r, Bp);
+    a.Tmax = Tmax;
     const bool ckpt = (flags & TDAGW_FLAG_CHECKPOINT) != 0;
     c.adj.valid = false;
     if (ckpt) {
@@ -675,11 +627,15 @@ void propagate_batched(Ctx& c, const tdagw_field* fields, int B, const int* step
         a.ckC = c.ckC.as<float2>();
         a.ck_period = period;
     }
+    const bool test_timeout = (flags & TDAGW_FLAG_TEST_TIMEOUT) != 0;
     if (test_timeout) {
         a.extra_arrivals = 1;
         a.wait_ns = 20000000ull;
     }
-    run(plan, Tmax);
+    launch_batched(c, fn, dim3(G), dim3(kBThreads), smem, &a, sizeof(a),
+                   {{c.bX.p, sbytes}, {c.bS.p, sbytes}, {c.bC.p, sbytes}, {c.sync.p, 4 * sizeof(unsigned)}},
+                   !(flags & TDAGW_FLAG_NO_GRAPH) && !test_timeout);
+    c.persistent_launched = true;
     a.extra_arrivals = 0;
     a.wait_ns = 2000000000ull;
     if (ckpt) {
@@ -689,8 +645,7 @@ void propagate_batched(Ctx& c, const tdagw_field* fields, int B, const int* step
         st.Bp = Bp;
         st.Tmax = Tmax;
         st.period = a.ck_period;
-        st.Rg = plan.Rg;
-        st.Tg = plan.Tg;
+        st.G = G;
         st.mode = mode;
         st.dt = dt;
         st.perm = perm;
@@ -701,8 +656,6 @@ void propagate_batched(Ctx& c, const tdagw_field* fields, int B, const int* step
         std::memcpy(st.fwd_args.data(), &a, sizeof(BatchArgs));
         st.fwd_fn = fn;
     }
-    c.last_plan_rg = plan.Rg;
-    c.last_plan_tg = plan.Tg;
     // observables in the caller's trajectory order
     finish_batch(c, bs, B);
 }
@@ -712,9 +665,7 @@ void propagate_batched(Ctx& c, const tdagw_field* fields, int B, const int* step
 namespace tdagw {
 
 // The backward sweep of the adjoint after a checkpointed split-FP16 (tensor-core) forward
-// run uses the FP32 batched partition: the low-rank plan cached for this batch size and
-// rank, else the first candidate shape (at most kTileB trajectories per block, CTAs <=
-// SMs).  Fills c.adj like a checkpointed FP32 run; the caller adds the tensor-core fields.
+// run uses the FP32 batched kernels' split (step_plan).  Fills c.adj like a checkpointed FP32 run; the caller adds the tensor-core fields.
 void prepare_adjoint_fp32(Ctx& c, const BatchSetup& bs, const tdagw_field* fields, int B, const int* steps,
                           double dt, int flags) {
     const HostModel& h = c.hm;
@@ -724,27 +675,14 @@ void prepare_adjoint_fp32(Ctx& c, const BatchSetup& bs, const tdagw_field* field
     int dev = 0, nsm = 0;
     TDAGW_CUDA(cudaGetDevice(&dev));
     TDAGW_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    const size_t smem = (size_t)kGemmSmem * sizeof(float2) +
-                        (size_t)(kBThreads / kTileB) * kTileB * 3 * sizeof(double);
+    const size_t smem = kBatchSmem;
     const void* fn = h.Nb == 2 ? (const void*)batched_kernel<2, false> : (const void*)batched_kernel<4, false>;
     TDAGW_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     TDAGW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBThreads, smem));
     TDAGW_REQUIRE(per_sm >= 1, TDAGW_ERR_UNSUPPORTED, "batched kernel does not fit on this device");
-    const int max_ctas = nsm * per_sm;
-    const uint64_t key = ((uint64_t)TDAGW_LOWRANK << 56) | ((uint64_t)B << 32) | (uint64_t)(uint32_t)r;
-    const int tg_min = (B + kTileB - 1) / kTileB;
-    BatchPlan plan;
-    auto it = c.batch_plans.find(key);
-    if (it != c.batch_plans.end() && it->second.second >= tg_min && it->second.first >= 1 &&
-        it->second.first <= h.Nk && it->second.first * it->second.second <= max_ctas) {
-        plan.Rg = it->second.first;
-        plan.Tg = it->second.second;
-    } else {
-        plan.Tg = tg_min;
-        plan.Rg = std::min(h.Nk, max_ctas / tg_min);
-        TDAGW_REQUIRE(plan.Rg >= 1, TDAGW_ERR_UNSUPPORTED, "too many trajectories for one launch");
-    }
+    const int G = nsm;
+    TDAGW_REQUIRE((B + kTileB - 1) / kTileB <= G, TDAGW_ERR_UNSUPPORTED, "too many trajectories for one launch");
     BatchArgs a{};
     a.U = c.U.as<float2>();
     a.V = c.V.as<float2>();
@@ -782,23 +720,15 @@ void prepare_adjoint_fp32(Ctx& c, const BatchSetup& bs, const tdagw_field* field
     c.sync.ensure(4 * sizeof(unsigned));
     a.bar = reinterpret_cast<unsigned long long*>(c.sync.p);
     a.err = reinterpret_cast<int*>(c.sync.as<unsigned>() + 2);
-    a.Rg = plan.Rg;
-    a.Tg = plan.Tg;
     a.Tmax = bs.Tmax;
-    c.bP.ensure((size_t)std::max(1, plan.Rg * std::max(r, 1)) * Bp * sizeof(float2));
-    c.bY.ensure((size_t)std::max(r, 1) * Bp * sizeof(float2));
-    c.bred.ensure((size_t)plan.Rg * Bp * 3 * sizeof(double));
-    a.P = c.bP.as<float2>();
-    a.Y = c.bY.as<float2>();
-    a.red = c.bred.as<double>();
+    batch_buffers(c, a, G, r, Bp);
     AdjointState& st = c.adj;
     st = AdjointState{};
     st.valid = true;
     st.B = B;
     st.Bp = Bp;
     st.Tmax = bs.Tmax;
-    st.Rg = plan.Rg;
-    st.Tg = plan.Tg;
+    st.G = G;
     st.mode = TDAGW_LOWRANK;
     st.dt = dt;
     st.perm = bs.perm;

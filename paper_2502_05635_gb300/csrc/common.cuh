@@ -143,7 +143,7 @@ void build_host_model(const tdagw_model_desc& d, HostModel& hm);
 // What the adjoint needs from the last checkpointed batched propagation.
 struct AdjointState {
     bool valid = false;
-    int B = 0, Bp = 0, Tmax = 0, period = 1, Rg = 0, Tg = 0, mode = 0;
+    int B = 0, Bp = 0, Tmax = 0, period = 1, G = 0, mode = 0;  // G: CTAs of the FP32 launches
     double dt = 0.0;
     std::vector<int> perm, steps;          // sorted -> caller order; caller-order lengths
     std::vector<tdagw_field> fields;       // caller order
@@ -224,9 +224,9 @@ struct Ctx {
     bool persistent_launched = false;
     // batched propagation: states N x Bp, intermediates, per-trajectory tables
     DevBuf bX, bS, bC, bA, bdS, bP, bY, bred, bobs, bEtab, bdir, bact, bperm, bfield, bchm;
-    // (mode << 56 | B << 32 | rank) -> (row groups, traj groups); B <= 65536, rank < 2^32
+    // tuned work split of the tensor-core launches: (kind << 56 | B << 32 | rank) -> split;
+    // B <= 65536, rank < 2^32
     std::map<uint64_t, std::pair<int, int>> batch_plans;
-    int last_plan_rg = 0, last_plan_tg = 0;
     int obs_B = 1;           // trajectories in the recorded observables
     // split-FP16 tiled factors for the tensor-core batched path, its intermediates, and
     // whether the tiles match the installed factors
