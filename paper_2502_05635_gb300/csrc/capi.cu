@@ -123,7 +123,7 @@ template <typename R> void build(Ctx& c) {
         b->ensure(N * sizeof(cplx_t<R>));
         TDAGW_CUDA(cudaMemsetAsync(b->p, 0, N * sizeof(cplx_t<R>), s));
     }
-    const int64_t blocks = (N + 255) / 256;
+    const int64_t blocks = (N + 31) / 32;  // the stage kernels' smallest blocks
     c.red.ensure(blocks * 3 * sizeof(double));
     c.counter.ensure(sizeof(unsigned));
     TDAGW_CUDA(cudaMemsetAsync(c.counter.p, 0, sizeof(unsigned), s));
@@ -239,14 +239,9 @@ template <typename R> void apply(Ctx& c, int mode, const void* x, void* y, cudaS
     } else {
         const int r = c.rank;
         const int64_t ldu = r + (r & 1);
-        launch_vcols<R>(c.V.p, ldu, N, r, x, c.ypart.p, c.ysplit, s);
-        launch_yreduce<R>(c.ypart.p, c.ysplit, r, c.S.p, c.ytil.p, s);
-        if (c.kdiag) {
-            launch_gemv<R>(c.U.p, ldu, N, r, c.ytil.p, y, 1, nullptr, nullptr, s);
-            launch_kblock_add<R>(c.kblkF.p, x, y, c.hm.Nk, c.hm.Nb * c.hm.Nb, s);
-        } else {
-            launch_gemv<R>(c.U.p, ldu, N, r, c.ytil.p, y, 1, c.diagF.p, x, s);
-        }
+        launch_lowrank_apply<R>(c.U.p, c.V.p, ldu, N, r, c.S.p, c.kdiag ? nullptr : c.diagF.p, x, y, c.ypart.p,
+                                c.ysplit, c.ytil.p, s);
+        if (c.kdiag) launch_kblock_add<R>(c.kblkF.p, x, y, c.hm.Nk, c.hm.Nb * c.hm.Nb, s);
     }
 }
 

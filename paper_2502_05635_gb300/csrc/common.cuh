@@ -282,6 +282,12 @@ void launch_vcols(const void* V, int64_t ldv, int64_t N, int r, const void* x, v
 template <typename R>
 void launch_yreduce(const void* part, int nsplit, int r, const void* S, void* ytil,
                     cudaStream_t s);
+// y = diag o x + U (S o (V^H x)) (diag nullptr: without): one cluster launch for small N r,
+// else the V pass into nblocks partial vectors (part, nblocks x r), their sum (ytil, r) and the
+// U pass.  U and V rows start on 16 bytes (even ld).
+template <typename R>
+void launch_lowrank_apply(const void* U, const void* V, int64_t ld, int64_t N, int r, const void* S, const void* diag,
+                          const void* x, void* y, void* part, int nblocks, void* ytil, cudaStream_t s);
 template <typename R>
 void launch_stage(Ctx& c, int stage, double dt, double dirx, double diry, bool kahan,
                   cudaStream_t s);

@@ -2,12 +2,18 @@
 // streaming complex GEMV (dense form of Eq. sigma-from-k, and the two passes of the
 // truncated-SVD form of Eq. svd_acc), and the fused per-k commutator + RK4 stage update +
 // observables kernel (Eq. tdagw).
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 #include "stage.cuh"
 
 namespace tdagw {
 
 namespace {
+
+// threads per block of the stage and observables kernels: in FP64 small blocks, which spread a
+// few thousand elements over the SMs (bound by the few FP64 pipes of each)
+template <typename R> constexpr int kStageThreads = sizeof(R) == 8 ? 32 : 256;
 
 // ---------------------------------------------------------------- vector loads -------
 
@@ -21,6 +27,15 @@ __device__ __forceinline__ void ld2_stream(const float2* p, float2& a, float2& b
 __device__ __forceinline__ void ld2_stream(const double2* p, double2& a, double2& b) {
     a = __ldcs(p);
     b = __ldcs(p + 1);
+}
+__device__ __forceinline__ void ld2_plain(const float2* p, float2& a, float2& b) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    a = make_float2(v.x, v.y);
+    b = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void ld2_plain(const double2* p, double2& a, double2& b) {
+    a = p[0];
+    b = p[1];
 }
 __device__ __forceinline__ void ld2_cached(const float2* p, float2& a, float2& b) {
     const float4 v = __ldg(reinterpret_cast<const float4*>(p));
@@ -132,15 +147,183 @@ vcols_kernel(const cplx_t<R>* __restrict__ V, int64_t ldv, int64_t N, int r,
     if (c + 1 < r) part[(int64_t)blockIdx.x * r + c + 1] = a1;
 }
 
-// ytil[j] = S[j] * sum_s part[s][j]: finishes y = S o (V^H x) of Eq. svd_acc.
+// ytil[j] = S[j] * sum_s part[s][j]: finishes y = S o (V^H x) of Eq. svd_acc.  kYCols columns
+// per block (128 or 256 contiguous bytes), the partials split over the rest of the threads (four
+// loads in flight each) and combined in a fixed order: one thread per column took a chain of
+// up to 304 loads (about 50 us).  Narrow blocks in FP64, whose additions would otherwise queue
+// at the pipes of a few SMs.
+constexpr int kYThreads = 512;
+template <typename R> constexpr int kYCols = sizeof(R) == 8 ? 8 : 32;
 template <typename R>
-__global__ void yreduce_kernel(const cplx_t<R>* __restrict__ part, int nsplit, int r,
-                               const R* __restrict__ S, cplx_t<R>* __restrict__ ytil) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= r) return;
-    cplx_t<R> s = part[j];
-    for (int q = 1; q < nsplit; ++q) s = cadd(s, part[(int64_t)q * r + j]);
-    ytil[j] = cscale(s, S[j]);
+__global__ void __launch_bounds__(kYThreads)
+yreduce_kernel(const cplx_t<R>* __restrict__ part, int nsplit, int r, const R* __restrict__ S,
+               cplx_t<R>* __restrict__ ytil) {
+    using C = cplx_t<R>;
+    constexpr int cols = kYCols<R>, subs = kYThreads / cols;
+    const int col = threadIdx.x % cols, sub = threadIdx.x / cols;
+    const int j = blockIdx.x * cols + col;
+    const int q0 = (int)((int64_t)sub * nsplit / subs), q1 = (int)((int64_t)(sub + 1) * nsplit / subs);
+    __shared__ C red[subs][cols];
+    C s[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s[u] = mk((R)0, (R)0);
+    if (j < r) {
+        int q = q0;
+        for (; q + 4 <= q1; q += 4) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) s[u] = cadd(s[u], part[(int64_t)(q + u) * r + j]);
+        }
+        for (; q < q1; ++q) s[0] = cadd(s[0], part[(int64_t)q * r + j]);
+    }
+    red[sub][col] = cadd(cadd(s[0], s[1]), cadd(s[2], s[3]));
+#pragma unroll
+    for (int o = subs / 2; o > 0; o >>= 1) {
+        __syncthreads();
+        if (sub < o) red[sub][col] = cadd(red[sub][col], red[sub + o][col]);
+    }
+    if (sub == 0 && j < r) ytil[j] = cscale(red[0][col], S[j]);
+}
+
+// Sums of W rows held one partial per lane: W 2^k halvings across the lanes, then plain
+// butterflies, so that four rows cost 6 complex additions per lane instead of 20 (FP64
+// additions are as dear as FMAs here).  The sum of row (lane >> (5 - log2 W)) is in every lane
+// of its group.
+template <int W, typename C> __device__ __forceinline__ C warp_rows_sum(C (&v)[W], int lane) {
+    int o = 16;
+#pragma unroll
+    for (int w = W; w > 1; w >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int q = 0; q < w / 2; ++q) {
+            const C keep = up ? v[q + w / 2] : v[q], send = up ? v[q] : v[q + w / 2];
+            v[q] = cadd(keep, shfl_xor(send, o));
+        }
+    }
+    C s = v[0];
+#pragma unroll
+    for (; o > 0; o >>= 1) s = cadd(s, shfl_xor(s, o));
+    return s;
+}
+
+// one warp's dot products of W consecutive rows of A (row stride lda) with x over ncols
+// columns, two complex per lane and step (rows and x start on 16 bytes)
+template <typename R, int W>
+__device__ __forceinline__ void row_dots(const cplx_t<R>* __restrict__ A, int64_t lda, int nrows, int ncols,
+                                         const cplx_t<R>* x, int lane, cplx_t<R> (&acc)[W]) {
+    using C = cplx_t<R>;
+#pragma unroll
+    for (int w = 0; w < W; ++w) acc[w] = mk((R)0, (R)0);
+    int c = 2 * lane;
+#pragma unroll 2
+    for (; c + 1 < ncols; c += 64) {
+        C x0, x1;
+        ld2_plain(x + c, x0, x1);
+#pragma unroll
+        for (int w = 0; w < W; ++w)
+            if (w < nrows) {
+                C a0, a1;
+                ld2_stream(A + w * lda + c, a0, a1);
+                acc[w] = cfma(a1, x1, cfma(a0, x0, acc[w]));
+            }
+    }
+    if (c < ncols) {
+        const C x0 = x[c];
+#pragma unroll
+        for (int w = 0; w < W; ++w)
+            if (w < nrows) acc[w] = cfma(A[w * lda + c], x0, acc[w]);
+    }
+}
+
+// out[row] = sum_c A[row, c] x[c] (+ diag[row] xd[row]), one warp per W rows: the U pass, whose
+// rows are short (a block of 256 threads per four rows left most of them idle below 512
+// columns and spent more on its reduction than on the products).
+template <typename R, int W>
+__global__ void __launch_bounds__(128)
+urows_kernel(const cplx_t<R>* __restrict__ A, int64_t lda, int64_t nrows, int ncols, const cplx_t<R>* __restrict__ x,
+             cplx_t<R>* __restrict__ out, const cplx_t<R>* __restrict__ diag, const cplx_t<R>* __restrict__ xd) {
+    using C = cplx_t<R>;
+    const int lane = threadIdx.x & 31;
+    const int64_t r0 = (blockIdx.x * (int64_t)4 + (threadIdx.x >> 5)) * W;
+    if (r0 >= nrows) return;
+    C acc[W];
+    row_dots<R, W>(A + r0 * lda, lda, (int)min((int64_t)W, nrows - r0), ncols, x, lane, acc);
+    C s = warp_rows_sum<W>(acc, lane);
+    const int64_t row = r0 + lane / (32 / W);
+    if (lane % (32 / W) == 0 && row < nrows) {
+        if (diag) s = cfma(diag[row], xd[row], s);
+        out[row] = s;
+    }
+}
+
+// ---------------------------------------------------------------- small apply --------
+
+// The whole low-rank application y = diag o x + U (S o (V^H x)) in one launch: one cluster of
+// eight CTAs, each with a contiguous share of the rows.  V^H x over the share (column pairs x
+// row subsets, subsets added in order), the eight partial vectors through distributed shared
+// memory, then the share's rows of U.  Bound by the three launches it replaces (small N r).
+constexpr int kClThreads = 512, kClCtas = 8, kClMaxRank = 512;
+// N r at most: N = 576, rank 29 takes 7.2 us a call (14.4 with three launches and the former
+// reductions), rank 110 10.3 (rank 120 with three launches 14.4); N = 2304, rank 28 12.3 (rank
+// 30 15.4).  Complex64 only: in complex128 eight SMs' FP64 pipes are slower than three launches.
+constexpr int64_t kClMaxElems = 65536;
+template <typename R>
+__global__ void __cluster_dims__(kClCtas, 1, 1) __launch_bounds__(kClThreads)
+lr_cluster_kernel(const cplx_t<R>* __restrict__ U, const cplx_t<R>* __restrict__ V, int64_t ld, int N, int r,
+                  const R* __restrict__ S, const cplx_t<R>* __restrict__ diag, const cplx_t<R>* __restrict__ x,
+                  cplx_t<R>* __restrict__ y) {
+    using C = cplx_t<R>;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ __align__(16) C sub[2 * kClThreads];
+    __shared__ __align__(16) C part[kClMaxRank], ys[kClMaxRank];
+    const int tid = threadIdx.x, lane = tid & 31, cta = (int)cl.block_rank();
+    const int i0 = (int)((int64_t)cta * N / kClCtas), i1 = (int)((int64_t)(cta + 1) * N / kClCtas);
+    const int ncp = (r + 1) / 2, nsub = kClThreads / ncp;
+    const int cp = tid % ncp, sb = tid / ncp;
+    C a0 = mk((R)0, (R)0), a1 = a0;
+    const bool two = 2 * cp + 1 < r;
+    if (sb < nsub) {
+#pragma unroll 4
+        for (int i = i0 + sb; i < i1; i += nsub) {
+            const C* v = V + i * ld + 2 * cp;
+            const C xi = x[i];
+            if (two) {
+                C v0, v1;
+                ld2_stream(v, v0, v1);
+                a0 = cfmac(v0, xi, a0);
+                a1 = cfmac(v1, xi, a1);
+            } else {
+                a0 = cfmac(v[0], xi, a0);
+            }
+        }
+        sub[2 * tid] = a0;
+        sub[2 * tid + 1] = a1;
+    }
+    __syncthreads();
+    for (int j = tid; j < r; j += kClThreads) {
+        C s = sub[j];
+        for (int u = 1; u < nsub; ++u) s = cadd(s, sub[2 * u * ncp + j]);
+        part[j] = s;
+    }
+    cl.sync();
+    for (int j = tid; j < r; j += kClThreads) {
+        C s = cl.map_shared_rank(part, 0)[j];
+#pragma unroll
+        for (int c = 1; c < kClCtas; ++c) s = cadd(s, cl.map_shared_rank(part, c)[j]);
+        ys[j] = cscale(s, S[j]);
+    }
+    cl.sync();  // the partials are read before any CTA exits; ys is complete
+    constexpr int W = 2;
+    for (int r0 = i0 + W * (tid >> 5); r0 < i1; r0 += W * (kClThreads / 32)) {
+        C acc[W];
+        row_dots<R, W>(U + r0 * ld, ld, min(W, i1 - r0), r, ys, lane, acc);
+        C s = warp_rows_sum<W>(acc, lane);
+        const int row = r0 + lane / (32 / W);
+        if (lane % (32 / W) == 0 && row < i1) {
+            if (diag) s = cfma(diag[row], x[row], s);
+            y[row] = s;
+        }
+    }
 }
 
 // ---------------------------------------------------------------- stage --------------
@@ -179,19 +362,39 @@ __device__ void reduce_observables(double v0, double v1, double v2, double* red,
         last = (t == gridDim.x - 1);
     }
     __syncthreads();
-    if (last && threadIdx.x == 0) {
+    if (last) {
+        // the last block's threads share the blocks' partials (fixed order); one thread alone
+        // waited for every one of them in turn
         __threadfence();
         double a = 0, b = 0, c = 0;
-        for (unsigned q = 0; q < gridDim.x; ++q) {
-            a += ((volatile double*)red)[q * 3 + 0];
-            b += ((volatile double*)red)[q * 3 + 1];
-            c += ((volatile double*)red)[q * 3 + 2];
+        for (unsigned q = threadIdx.x; q < gridDim.x; q += blockDim.x) {
+            a += __ldcg(red + q * 3 + 0);
+            b += __ldcg(red + q * 3 + 1);
+            c += __ldcg(red + q * 3 + 2);
         }
-        obs_row[0] = a * inv_nk;
-        obs_row[1] = b * inv_nk;
-        obs_row[2] = c * inv_nk;
-        *counter = 0u;
-        if (step_to_bump) *step_to_bump = new_step;
+        for (int o = 16; o > 0; o >>= 1) {
+            a += __shfl_xor_sync(0xffffffffu, a, o);
+            b += __shfl_xor_sync(0xffffffffu, b, o);
+            c += __shfl_xor_sync(0xffffffffu, c, o);
+        }
+        if (lane == 0) {
+            sred[warp][0] = a;
+            sred[warp][1] = b;
+            sred[warp][2] = c;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
+                a += sred[w][0];
+                b += sred[w][1];
+                c += sred[w][2];
+            }
+            obs_row[0] = a * inv_nk;
+            obs_row[1] = b * inv_nk;
+            obs_row[2] = c * inv_nk;
+            *counter = 0u;
+            if (step_to_bump) *step_to_bump = new_step;
+        }
     }
 }
 
@@ -203,7 +406,7 @@ __device__ void reduce_observables(double v0, double v1, double v2, double* red,
 // the Nb^2 threads of one k are adjacent lanes of a warp and exchange the Nb x Nb blocks
 // by shuffles.
 template <typename R, int NB>
-__global__ void __launch_bounds__(256) stage_kernel(StageParams<R> p) {
+__global__ void __launch_bounds__(kStageThreads<R>) stage_kernel(StageParams<R> p) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t nstep = *p.step;
     const int eoff = p.stage == 0 ? 0 : (p.stage == 3 ? 2 : 1);
@@ -217,7 +420,7 @@ __global__ void __launch_bounds__(256) stage_kernel(StageParams<R> p) {
 
 // Observables of rho0 + X into obs row `row` (used for the initial row of a run).
 template <typename R, int NB>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kStageThreads<R>)
 observables_kernel(const cplx_t<R>* __restrict__ X, const cplx_t<R>* __restrict__ dx,
                    const cplx_t<R>* __restrict__ vx, int64_t N, int Nk, int c1, R o0_, R o1_,
                    R o2_, R o3_, double* red, unsigned* counter, double* obs_row) {
@@ -314,10 +517,40 @@ template <typename R>
 void launch_yreduce(const void* part, int nsplit, int r, const void* S, void* ytil,
                     cudaStream_t s) {
     using C = cplx_t<R>;
-    yreduce_kernel<R><<<(r + 255) / 256, 256, 0, s>>>(static_cast<const C*>(part), nsplit, r,
+    yreduce_kernel<R><<<(r + kYCols<R> - 1) / kYCols<R>, kYThreads, 0, s>>>(static_cast<const C*>(part), nsplit, r,
                                                        static_cast<const R*>(S),
                                                        static_cast<C*>(ytil));
     check_launch("yreduce_kernel");
+}
+
+template <typename R>
+void launch_urows(const void* A, int64_t lda, int64_t nrows, int ncols, const void* x, void* out, const void* diag,
+                  const void* xd, cudaStream_t s) {
+    using C = cplx_t<R>;
+    // one row per warp while that leaves SMs without a block
+    const bool few = nrows < 4 * 4 * 152;
+    const int64_t rpb = few ? 4 : 16;
+    auto k = few ? urows_kernel<R, 1> : urows_kernel<R, 4>;
+    k<<<(unsigned)((nrows + rpb - 1) / rpb), 128, 0, s>>>(static_cast<const C*>(A), lda, nrows, ncols,
+                                                          static_cast<const C*>(x), static_cast<C*>(out),
+                                                          static_cast<const C*>(diag), static_cast<const C*>(xd));
+    check_launch("urows_kernel");
+}
+
+template <typename R>
+void launch_lowrank_apply(const void* U, const void* V, int64_t ld, int64_t N, int r, const void* S, const void* diag,
+                          const void* x, void* y, void* part, int nblocks, void* ytil, cudaStream_t s) {
+    using C = cplx_t<R>;
+    if (sizeof(R) == 4 && r <= kClMaxRank && N * r <= kClMaxElems) {
+        lr_cluster_kernel<R><<<kClCtas, kClThreads, 0, s>>>(
+            static_cast<const C*>(U), static_cast<const C*>(V), ld, (int)N, r, static_cast<const R*>(S),
+            static_cast<const C*>(diag), static_cast<const C*>(x), static_cast<C*>(y));
+        check_launch("lr_cluster_kernel");
+        return;
+    }
+    launch_vcols<R>(V, ld, N, r, x, part, nblocks, s);
+    launch_yreduce<R>(part, nblocks, r, S, ytil, s);
+    launch_urows<R>(U, ld, N, r, ytil, y, diag, x, s);
 }
 
 template <typename R>
@@ -349,24 +582,24 @@ void launch_stage(Ctx& c, int stage, double dt, double dirx, double diry, bool k
     p.diry = (R)diry;
     p.stage = stage;
     p.kahan = kahan ? 1 : 0;
-    const unsigned blocks = (unsigned)((c.hm.N + 255) / 256);
-    if (c.hm.Nb == 2) stage_kernel<R, 2><<<blocks, 256, 0, s>>>(p);
-    else stage_kernel<R, 4><<<blocks, 256, 0, s>>>(p);
+    const unsigned blocks = (unsigned)((c.hm.N + kStageThreads<R> - 1) / kStageThreads<R>);
+    if (c.hm.Nb == 2) stage_kernel<R, 2><<<blocks, kStageThreads<R>, 0, s>>>(p);
+    else stage_kernel<R, 4><<<blocks, kStageThreads<R>, 0, s>>>(p);
     check_launch("stage_kernel");
 }
 
 template <typename R>
 void launch_observables_row(Ctx& c, const void* X, int64_t row, cudaStream_t s) {
     using C = cplx_t<R>;
-    const unsigned blocks = (unsigned)((c.hm.N + 255) / 256);
+    const unsigned blocks = (unsigned)((c.hm.N + kStageThreads<R> - 1) / kStageThreads<R>);
     const HostModel& h = c.hm;
     double* orow = c.obs.as<double>() + row * 3;
     if (h.Nb == 2)
-        observables_kernel<R, 2><<<blocks, 256, 0, s>>>(
+        observables_kernel<R, 2><<<blocks, kStageThreads<R>, 0, s>>>(
             static_cast<const C*>(X), c.dx.as<C>(), c.vx.as<C>(), h.N, h.Nk, h.c1, (R)h.occ[0],
             (R)h.occ[1], (R)h.occ[2], (R)h.occ[3], c.red.as<double>(), c.counter.as<unsigned>(), orow);
     else
-        observables_kernel<R, 4><<<blocks, 256, 0, s>>>(
+        observables_kernel<R, 4><<<blocks, kStageThreads<R>, 0, s>>>(
             static_cast<const C*>(X), c.dx.as<C>(), c.vx.as<C>(), h.N, h.Nk, h.c1, (R)h.occ[0],
             (R)h.occ[1], (R)h.occ[2], (R)h.occ[3], c.red.as<double>(), c.counter.as<unsigned>(), orow);
     check_launch("observables_kernel");
@@ -378,6 +611,8 @@ void launch_observables_row(Ctx& c, const void* X, int64_t row, cudaStream_t s) 
     template void launch_yreduce<R>(const void*, int, int, const void*, void*, cudaStream_t); \
     template void launch_vcols<R>(const void*, int64_t, int64_t, int, const void*, void*, int, \
                                   cudaStream_t);                                          \
+    template void launch_lowrank_apply<R>(const void*, const void*, int64_t, int64_t, int, const void*, const void*, \
+                                          const void*, void*, void*, int, void*, cudaStream_t); \
     template void launch_stage<R>(Ctx&, int, double, double, double, bool, cudaStream_t);   \
     template void launch_observables_row<R>(Ctx&, const void*, int64_t, cudaStream_t);
 INST(float)

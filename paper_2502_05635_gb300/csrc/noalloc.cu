@@ -98,9 +98,7 @@ extern "C" int tdagw_apply_lowrank_noalloc(const void* U, const void* V, int64_t
         // every partial entry and every used entry of ytil is written before it is read,
         // so nothing in the shared scratch has to be cleared between calls
         const int nblocks = (int)(N < kNoallocBlocks ? N : kNoallocBlocks);
-        launch_vcols<float>(V, ld, N, rank, x, part, nblocks, s);
-        launch_yreduce<float>(part, nblocks, rank, S, ytil, s);
-        launch_gemv<float>(U, ld, N, rank, ytil, y, 1, diag, x, s);
+        launch_lowrank_apply<float>(U, V, ld, N, rank, S, diag, x, y, part, nblocks, ytil, s);
         last_error_message().clear();
         return TDAGW_OK;
     } catch (const Error& e) {
