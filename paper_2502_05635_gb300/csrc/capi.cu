@@ -277,7 +277,10 @@ template <typename R> void propagate(Ctx& c, const tdagw_field& f, int T, double
     const double dirx = f.dir_x, diry = f.dir_y;
     int done = 0;
     const bool test_timeout = (flags & TDAGW_FLAG_TEST_TIMEOUT) != 0;
-    if (mode == TDAGW_LOWRANK && !(flags & TDAGW_FLAG_STAGEWISE) && T > 0 &&
+    if ((mode == TDAGW_LOWRANK || mode == TDAGW_FULL) && !(flags & TDAGW_FLAG_STAGEWISE) && T > 0 &&
+        launch_resident(c, mode, T, dt, dirx, diry, kahan, test_timeout, s))
+        done = T;
+    if (mode == TDAGW_LOWRANK && done == 0 && !(flags & TDAGW_FLAG_STAGEWISE) && T > 0 &&
         launch_lr_persistent(c, T, dt, dirx, diry, kahan, test_timeout, s))
         done = T;
     if (mode == TDAGW_CHANNEL && !(flags & TDAGW_FLAG_STAGEWISE) && T > 0 &&

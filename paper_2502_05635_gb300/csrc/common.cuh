@@ -356,6 +356,11 @@ void tc_recompute_segment(Ctx& c, int n0, int len, float2* recX, float2* recDS, 
 bool launch_lr_persistent(Ctx& c, int T, double dt, double dirx, double diry, bool kahan,
                           bool test_timeout, cudaStream_t s);
 
+// Persistent single-trajectory propagation with the kernel (dense or low rank) resident in shared
+// memory (small models, complex64); false if not applicable.
+bool launch_resident(Ctx& c, int mode, int T, double dt, double dirx, double diry, bool kahan, bool test_timeout,
+                     cudaStream_t s);
+
 template <typename R>
 void rsvd_compress(Ctx& c, int rank, int oversample, int power_iters, uint64_t seed);
 
