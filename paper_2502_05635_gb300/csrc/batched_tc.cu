@@ -84,12 +84,9 @@ constexpr uint32_t kLbo = 128, kSbo = (kKc / 8) * 128;
 constexpr uint32_t kStg = 32768;           // staged quarter tile: 64 rows x 64 trajectories
 constexpr int kTmemCols = 512;
 constexpr uint32_t kAcol = 256;            // tensor-memory columns of the operand blocks
-// The workers read the values of each operand block (16 rows of X or of S o Y for their
-// trajectories) through shared memory: asynchronous copies issued kSrcAhead chunks ahead
-// into kSrcSlots slots of 8 KB (the staging buffer of the epilogue, idle while the
-// operands stream), so the block builds do not wait on L2 latency.
-constexpr int kSrcSlots = 4, kSrcAhead = 3;
-static_assert(kSrcSlots * 8192 <= (int)32768 && kSrcAhead < kSrcSlots, "operand source slots");
+// source slots of the workers' operand values (two of 2 KB per warp, in the staging buffer of
+// the epilogue, idle while the operands stream)
+static_assert(kWorkers / 32 * 2 * 2048 <= (int)kStg, "operand source slots");
 static_assert(kRing >= 2 && kRing < kCmb, "ring depth");
 static_assert(kAcol + 32 * kAbuf <= (uint32_t)kTmemCols, "tensor memory");
 #ifndef TDAGW_TC_EVICT_FIRST
@@ -478,7 +475,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) batched_tc_kernel(TcArgs a) {
     const bool in_sync = warp >= 1;  // grid-barrier participants (lanes 1-31 of warp 0 idle)
     const int wt = tid - 64;  // worker index
     // worker warps: tensor-memory lane quarter (rows 32 q .. 32 q + 31 of the operand and of
-    // the accumulator) and half (which columns of a block the warp writes or reads)
+    // the accumulator) and half (which chunks the warp builds, which accumulator columns it reads)
     const int wq = warp & 3, wh = (warp - 2) >> 2;
     const int orow = 32 * wq + lane;           // operand / accumulator row: 2 bl + comp
     const int obl = orow >> 1, ocomp = orow & 1;
@@ -493,7 +490,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) batched_tc_kernel(TcArgs a) {
         abort_s = 0;
         for (int s = 0; s < kRing; ++s) mbar_init(full + s, 1);
         for (int s = 0; s < kCmb; ++s) mbar_init(cmb + s, 1);
-        for (int s = 0; s < kAbuf; ++s) mbar_init(afull + s, kWorkers / 32);
+        for (int s = 0; s < kAbuf; ++s) mbar_init(afull + s, kWorkers / 64);  // one set of worker warps
         mbar_init(accf, 1);
         mbar_init(acce, kWorkers);
         mbar_init(fin, 1);
@@ -511,9 +508,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) batched_tc_kernel(TcArgs a) {
     uint32_t acnt = 0;  // uses of the accumulator (MMA thread and workers)
     int gch = 0;        // chunks so far (all roles count the same sequence)
     int slot_ch[kRing]; // producer: chunk that last used each ring slot
-    int buf_ch[kAbuf];  // workers: chunk that last used each operand block
     for (int q = 0; q < kRing; ++q) slot_ch[q] = -1;
-    for (int q = 0; q < kAbuf; ++q) buf_ch[q] = -1;
     unsigned gen = 0;
     bool ok = true;
     unsigned long long tdone_target = 0;  // low-rank mode: epilogue items per tile so far
@@ -582,91 +577,83 @@ __global__ void __launch_bounds__(kTcThreads, 1) batched_tc_kernel(TcArgs a) {
         TC_W_END(a0, 2);
         tc::fence_after_sync();
     };
-    // workers: write the operand block of chunk gch into tensor memory: the warp's 32 rows
-    // (2 bl + comp), its 8 of the chunk's 16 complex columns, hi and lo parts.  v[u] is the
-    // (already scaled) complex value of column 8 wh + u; conj selects the expansion:
-    //   V^H X:  row 2b: (re, im), row 2b + 1: (im, -re)
-    //   U Y:    row 2b: (re, -im), row 2b + 1: (im, re)
-    auto build_block = [&](const float2 (&v)[8], bool vhx) {
-        const uint32_t bs = bu % kAbuf;
-        TC_W_BEGIN(w6);
-        if (!*vabort && !chunk_done(buf_ch[bs])) fail();
-        if (wt == 0) TC_W_END(w6, 6);
-        buf_ch[bs] = gch;
-        if (!warp_abort()) {
-            uint32_t hi[8], lo[8];
+    // workers: the operand blocks of chunks [c0, c1) of an item, in tensor memory.  The two
+    // sets of four warps (one warp per lane quarter) build alternate chunks, so that a set has
+    // two chunks' time for its chain of copy, conversion and tensor-memory store: the chain,
+    // not the instruction rate, bounded the builds when all eight warps shared every chunk
+    // (precision-study size, 12 steps: 13.6 -> 12.7 ms; channel-wise mos2 size, B = 64, 30
+    // steps: 22.9 -> 19.0 ms).  A lane
+    // writes row 2 bl + comp: the 16 complex columns of the chunk, hi and lo parts, expanded as
+    //   V^H X (vhx):  row 2b: (re, im), row 2b + 1: (im, -re)
+    //   U Y:          row 2b: (re, -im), row 2b + 1: (im, re)
+    // The source values come through shared memory: asynchronous copies one own chunk ahead
+    // into two slots of 2 KB per warp (16 trajectories x 16 values, columns XOR-swizzled by
+    // trajectory against bank conflicts); each lane of a pair copies 8 of the pair's 16 values.
+    // copies(c, dst): issue the lane's copies of chunk c (element j of its 8 to dst(j)).
+    float2* srcbuf = sDS + (warp - 2) * 512;
+    auto src_at = [&](int slot, int u) -> float2* { return srcbuf + slot * 256 + (obl & 15) * 16 + (u ^ (obl & 15)); };
+    auto build_chunks = [&](int c0, int c1, float sc, bool vhx, auto copies) {
+        auto issue = [&](int c, int slot) {
+            if (c < c1) copies(c, slot);
+            cp_async_commit();
+        };
+        issue(c0 + wh, 0);
+        int slot = 0;
+        for (int c = c0; c < c1; ++c, ++gch, ++bu) {
+            if (((c - c0) & 1) != wh) continue;
+            issue(c + 2, slot ^ 1);
+            const uint32_t bs = bu % kAbuf;
+            TC_W_BEGIN(w7);
+            cp_async_wait<1>();
+            __syncwarp();
+            if (wt == 0) TC_W_END(w7, 7);
+            TC_W_BEGIN(w6);
+            // the operand block is free once the chunk kAbuf before this one is complete
+            if (!*vabort && !chunk_done(gch - kAbuf)) fail();
+            if (wt == 0) TC_W_END(w6, 6);
+            if (!warp_abort()) {
+                const uint32_t ta = tm + ((uint32_t)(32 * wq) << 16) + kAcol + 32 * bs;
+#pragma unroll 1
+                for (int half = 0; half < 2; ++half) {
+                    uint32_t hi[8], lo[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                float p0, p1;
-                if (vhx) {
-                    p0 = ocomp ? v[u].y : v[u].x;
-                    p1 = ocomp ? -v[u].x : v[u].y;
-                } else {
-                    p0 = ocomp ? v[u].y : v[u].x;
-                    p1 = ocomp ? v[u].x : -v[u].y;
+                    for (int u = 0; u < 8; ++u) {
+                        const float2 x = *src_at(slot, 8 * half + u);
+                        const float re = x.x * sc, im = x.y * sc;
+                        const float p0 = ocomp ? im : re;
+                        const float p1 = vhx ? (ocomp ? -re : im) : (ocomp ? re : -im);
+                        // split both values at once: hi = fp16(p), lo = fp16(p - hi)
+                        const __half2 h = __floats2half2_rn(p0, p1);
+                        const float2 hb = __half22float2(h);
+                        const __half2 l = __floats2half2_rn(p0 - hb.x, p1 - hb.y);
+                        hi[u] = *reinterpret_cast<const uint32_t*>(&h);
+                        lo[u] = *reinterpret_cast<const uint32_t*>(&l);
+                    }
+                    tc::tmem_st8_nowait(ta + 8 * half, hi);
+                    tc::tmem_st8_nowait(ta + 16 + 8 * half, lo);
                 }
-                // split both values at once (paired conversions): hi = fp16(p), lo = fp16(p - hi)
-                const __half2 h = __floats2half2_rn(p0, p1);
-                const float2 hb = __half22float2(h);
-                const __half2 l = __floats2half2_rn(p0 - hb.x, p1 - hb.y);
-                hi[u] = *reinterpret_cast<const uint32_t*>(&h);
-                lo[u] = *reinterpret_cast<const uint32_t*>(&l);
+                TC_W_BEGIN(w8);
+                tc::tmem_wait_st();
+                if (wt == 0) TC_W_END(w8, 8);
             }
-            const uint32_t ta = tm + ((uint32_t)(32 * wq) << 16) + kAcol + 32 * bs + 8 * wh;
-            TC_W_BEGIN(w8);
-            tc::tmem_st8(ta, hi);
-            tc::tmem_st8(ta + 16, lo);
-            if (wt == 0) TC_W_END(w8, 8);
+            tc::fence_before_sync();
+            __syncwarp();  // the slot may be refilled after every lane has read it
+            if (lane == 0) mbar_arrive(afull + bs);
+            slot ^= 1;
         }
-        tc::fence_before_sync();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(afull + bs);
-        ++bu;
-        ++gch;
+        cp_async_wait<0>();
     };
-
-    // workers: the source values of chunk c (rows 16 c .. 16 c + 15 of X or of S o Y, the
-    // warp's 8 of them, its 16 trajectories) into source slot k % kSrcSlots; each lane of
-    // a pair copies 4 of the pair's 8 values, one completion group per chunk (empty past
-    // the item's last chunk c_end).  Rows past N are zero-filled.
-    float2* srcbuf = sDS;  // kSrcSlots x 8 KB, warp part (warp - 2) x 1 KB
-    auto src_issue = [&](const float2* base, int c, int c_end, bool live, int b0, int k) {
-        if (c < c_end) {
-            float2* dst = srcbuf + (k % kSrcSlots) * 1024 + (warp - 2) * 128 + (obl & 15) * 8 + 4 * ocomp;
+    // the lane's 8 copies of chunk c from rows 16 c .. 16 c + 15 of base (rows from `rows` on
+    // are zero), row stride ldr; live: the lane has a trajectory (column col of the rows)
+    auto copy_rows = [&](const float2* base, int64_t ldr, int64_t rows, bool live, int c, int slot) {
+        const int64_t i0 = (int64_t)c * 16 + 8 * ocomp;
+        const float2* p = base + i0 * ldr;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int64_t i = (int64_t)c * 16 + 8 * wh + 4 * ocomp + u;
-                const bool v = live && i < a.N;
-                cp_async8(dst + u, v ? (const void*)(base + i * a.Bp + b0 + obl) : (const void*)base, v ? 8u : 0u);
-            }
+        for (int u = 0; u < 8; ++u) {
+            const bool v = live && i0 + u < rows;
+            cp_async8(src_at(slot, 8 * ocomp + u), v ? (const void*)p : (const void*)a.X, v ? 8u : 0u);
+            p += ldr;
         }
-        cp_async_commit();
-    };
-    // the same with the rows given by rowp(i): the row's base pointer, or null for a zero
-    // row (channel-wise mode: gathered rows of X and of S o Y)
-    auto src_issue_rows = [&](auto rowp, int c, int c_end, bool live, int b0, int k) {
-        if (c < c_end) {
-            float2* dst = srcbuf + (k % kSrcSlots) * 1024 + (warp - 2) * 128 + (obl & 15) * 8 + 4 * ocomp;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int64_t i = (int64_t)c * 16 + 8 * wh + 4 * ocomp + u;
-                const float2* row = live ? rowp(i) : nullptr;
-                cp_async8(dst + u, row ? (const void*)(row + b0 + obl) : (const void*)a.X, row ? 8u : 0u);
-            }
-        }
-        cp_async_commit();
-    };
-    // workers: wait for the source values of the chunk in slot k (kSrcAhead - 1 newer
-    // groups may stay in flight) and read the pair's 8 values, scaled
-    auto src_read = [&](float2 (&v)[8], int k, float sc) {
-        TC_W_BEGIN(w7);
-        cp_async_wait<kSrcAhead - 1>();
-        __syncwarp();
-        if (wt == 0) TC_W_END(w7, 7);
-        const float2* src = srcbuf + (k % kSrcSlots) * 1024 + (warp - 2) * 128 + (obl & 15) * 8;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = make_float2(src[u].x * sc, src[u].y * sc);
-        __syncwarp();  // the slot may be refilled after every lane has read it
     };
 
     for (int n = 0; n < a.Tmax && ok && (in_sync || producer); ++n) {
@@ -748,33 +735,19 @@ __global__ void __launch_bounds__(kTcThreads, 1) batched_tc_kernel(TcArgs a) {
                     workers_sync();
                     const float sx = ssc[obl];
                     const bool live = obl < nbg;
-                    // X values of the warp's columns of chunk c, kSrcAhead chunks ahead
                     if constexpr (CHT) {
                         // rows k' P + q of X for the V segment q of this item
                         int qs, m;
                         seg_of_mt(a, it.m, qs, m);
-                        const int P = a.npair, Nk = a.Nk;
-                        auto rowx = [&](int64_t i) -> const float2* {
-                            return i < Nk ? a.X + (i * P + qs) * a.Bp : nullptr;
-                        };
-                        for (int c = it.c0; c < it.c0 + kSrcAhead; ++c)
-                            src_issue_rows(rowx, c, it.c1, live, b0, c - it.c0);
-                        for (int c = it.c0; c < it.c1; ++c) {
-                            float2 v[8];
-                            src_read(v, c - it.c0, sx);
-                            build_block(v, true);
-                            src_issue_rows(rowx, c + kSrcAhead, it.c1, live, b0, c + kSrcAhead - it.c0);
-                        }
+                        const float2* xq = a.X + (int64_t)qs * a.Bp + b0 + obl;
+                        build_chunks(it.c0, it.c1, sx, true, [&](int c, int slot) {
+                            copy_rows(xq, (int64_t)a.npair * a.Bp, a.Nk, live, c, slot);
+                        });
                     } else {
-                        for (int c = it.c0; c < it.c0 + kSrcAhead; ++c) src_issue(a.X, c, it.c1, live, b0, c - it.c0);
-                        for (int c = it.c0; c < it.c1; ++c) {
-                            float2 v[8];
-                            src_read(v, c - it.c0, sx);
-                            build_block(v, true);
-                            src_issue(a.X, c + kSrcAhead, it.c1, live, b0, c + kSrcAhead - it.c0);
-                        }
+                        const float2* xb = a.X + b0 + obl;
+                        build_chunks(it.c0, it.c1, sx, true,
+                                     [&](int c, int slot) { copy_rows(xb, a.Bp, a.N, live, c, slot); });
                     }
-                    cp_async_wait<0>();
                     // accumulator -> raw partials P[ks][j][b]: lanes 2 bl and 2 bl + 1 hold the
                     // real and imaginary parts; the warp's half of the 256 columns (rows j)
                     if (!*vabort && !mb_wait(accf, acnt & 1u, vabort, budget)) fail();
@@ -941,15 +914,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) batched_tc_kernel(TcArgs a) {
                         }
                         workers_sync();
                         const bool live = obl < nbg;
-                        // S o Y values of the warp's columns of chunk c, kSrcAhead chunks ahead
-                        for (int c = 0; c < kSrcAhead; ++c) src_issue(a.Ys, c, a.nchU, live, b0, c);
-                        for (int c = 0; c < a.nchU; ++c) {
-                            float2 v[8];
-                            src_read(v, c, 1.f);
-                            build_block(v, false);
-                            src_issue(a.Ys, c + kSrcAhead, a.nchU, live, b0, c + kSrcAhead);
-                        }
-                        cp_async_wait<0>();
+                        const float2* yb = a.Ys + b0 + obl;
+                        build_chunks(0, a.nchU, 1.f, false,
+                                     [&](int c, int slot) { copy_rows(yb, a.Bp, a.N, live, c, slot); });
                         if (!*vabort && !mb_wait(accf, acnt & 1u, vabort, budget)) fail();
                         tc::fence_after_sync();
                         const int kgroups = kWorkers / nbg;
@@ -1071,18 +1038,22 @@ __global__ void __launch_bounds__(kTcThreads, 1) batched_tc_kernel(TcArgs a) {
                         // operand z_p: the S o y rows of the channels out of p, then x_p
                         const int nl = a.nlrq[p], P = a.npair, Nk = a.Nk;
                         const int* gp = a.gpad + a.gbq[p];
-                        auto rowz = [&](int64_t j) -> const float2* {
-                            if (j < nl) return a.Ys + (int64_t)__ldg(gp + j) * a.Bp;
-                            return j < nl + Nk ? a.X + ((j - nl) * P + p) * a.Bp : nullptr;
-                        };
-                        for (int c = c0; c < c0 + kSrcAhead; ++c) src_issue_rows(rowz, c, c1, live, b0, c - c0);
-                        for (int c = c0; c < c1; ++c) {
-                            float2 v[8];
-                            src_read(v, c - c0, sz);
-                            build_block(v, false);
-                            src_issue_rows(rowz, c + kSrcAhead, c1, live, b0, c + kSrcAhead - c0);
-                        }
-                        cp_async_wait<0>();
+                        const float2* xp = a.X + (int64_t)p * a.Bp + b0 + obl;
+                        build_chunks(c0, c1, sz, false, [&](int c, int slot) {
+                            if (c * 16 >= nl) {
+                                // rows of x_p: row j - nl of the strided x_p for the operand's row j
+                                copy_rows(xp - (int64_t)nl * P * a.Bp, (int64_t)P * a.Bp, (int64_t)nl + Nk, live, c, slot);
+                                return;
+                            }
+#pragma unroll 1
+                            for (int u = 0; u < 8; ++u) {
+                                const int j = c * 16 + 8 * ocomp + u;
+                                const float2* row = j < nl ? a.Ys + (int64_t)__ldg(gp + j) * a.Bp + b0 + obl
+                                                           : xp + (int64_t)(j - nl) * P * a.Bp;
+                                const bool v = live && j < nl + Nk;
+                                cp_async8(src_at(slot, 8 * ocomp + u), v ? (const void*)row : (const void*)a.X, v ? 8u : 0u);
+                            }
+                        });
                         // accumulator -> partial dSigma rows k P + p of K-range kc (unscaled);
                         // lanes 2 bl and 2 bl + 1 hold the real and imaginary parts
                         if (!*vabort && !mb_wait(accf, acnt & 1u, vabort, budget)) fail();
