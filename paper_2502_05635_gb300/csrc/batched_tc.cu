@@ -36,7 +36,7 @@
 // The channel-wise mode (Eq. svd-channel-wise, a second instantiation) runs phase A per V
 // segment and phase C per U segment (low-rank columns and the dense diagonal channel of an
 // output pair) with gathered operand rows, writes dSigma to global memory, and runs the
-// epilogue as a fourth phase by 64-row quarters, with grid barriers between all phases.
+// epilogue as a fourth phase over all k-points, with grid barriers between all phases.
 // Roles: warp 0 streams the factor tiles into the ring (it only reads static tiles, so it
 // stays out of the grid barriers and keeps copies in flight across them), warp 1 issues
 // the MMAs, warps 2-9 build the tensor-memory operands and drain the accumulator.  Every
@@ -139,7 +139,7 @@ struct TcArgs {
     float su, sv;   // power-of-two scales of the U and V tiles
     float ybound;   // max|S| max_j ||v_j|| sqrt(2N): |(S o Y)_jb| <= ybound max|X_b|
     unsigned long long wait_ns;
-    int Nred;       // tiles of the per-tile observable sums (red): row tiles, or quarters
+    int Nred;       // entries of the partial observable sums (red): row tiles, or CTAs
     int extra_arrivals;  // > 0 only for the timeout test: the grid barrier can never complete
     // low-rank mode: per 256-row tile, the epilogue items completed so far (monotonic) and
     // max(|Re|, |Im|) of the new stage input per trajectory (float bits): a phase A item
@@ -153,11 +153,10 @@ struct TcArgs {
     // U segments (segment p = [U^pq of the channels out of p | K^pp]: NtK 256-row tiles of
     // k-points, nchw[p] chunks of its columns), with the operand z_p = [S o y of those
     // channels (padded rows gpad) ; x_p]; phase C writes dSigma to dS (one partial slot per
-    // K-range) and a fourth phase runs the commutator + RK4 epilogue by 64-row quarters of
-    // the nte 256-row tiles of all N rows.
+    // K-range) and a fourth phase runs the commutator + RK4 epilogue of all k-points.
     const int* gpad;
     float2* dS;
-    int npair, NtK, nte;
+    int npair, NtK;
     int kcu;        // K-ranges of a U segment tile (partial dSigma slots dS + kc N Bp)
     float zbound;   // |z_p| <= zbound max|X_b|
     long long tvoff[kMaxPairs], tuoff[kMaxPairs];
@@ -294,8 +293,9 @@ struct DF3 {
 // the FP32 batched path), with the low-rank part of dSigma read from the staged quarter
 // tile (block rows row0 .. row0 + NB^2 - 1, trajectory column bl) and K^diag o X added here.
 // xm: running max(|Re|, |Im|) of the values written to X (the next stage input); ob: the
-// thread's running sums of the observables (last stage).
-template <int NB>
+// thread's running sums of the observables (last stage).  GDS (channel-wise mode): all of
+// dSigma from global memory, summed over the K-range partials of phase C in a fixed order.
+template <int NB, bool GDS>
 __device__ void stage_kb_tc(const TcArgs& a, int k, int b, int st, float E, float2 dr,
                             const float2* sDS, int row0, int bl, float& xm, DF3& ob, int64_t rec) {
     constexpr int NB2 = NB * NB;
@@ -306,7 +306,13 @@ __device__ void stage_kb_tc(const TcArgs& a, int k, int b, int st, float E, floa
         const int64_t i = (int64_t)k * NB2 + g;
         X[g] = __ldcg(a.X + i * Bp + b);
         const float2 d1 = a.dx[i], d2 = a.dy[i];
-        const float2 ds = cfma(a.diag[i], X[g], sDS[ds_index(row0 + g, bl)]);
+        float2 ds;
+        if (GDS) {
+            ds = __ldcg(a.dS + i * Bp + b);
+            for (int kc = 1; kc < a.kcu; ++kc) ds = cadd(ds, __ldcg(a.dS + ((int64_t)kc * a.N + i) * Bp + b));
+        } else {
+            ds = cfma(a.diag[i], X[g], sDS[ds_index(row0 + g, bl)]);
+        }
         if (rec >= 0) {  // stage input and dSigma, for the adjoint's backward sweep
             a.recX[rec + i * Bp + b] = X[g];
             a.recDS[rec + i * Bp + b] = ds;
@@ -951,7 +957,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) batched_tc_kernel(TcArgs a) {
                                 const float2 dr = a.dir[b];
                                 const int64_t rec = a.recX ? (int64_t)(4 * n + st) * a.N * a.Bp : -1;
                                 for (int kl = kg; kl < kt; kl += kgroups)
-                                    stage_kb_tc<NB>(a, kbase + kl, b, st, E, dr, sDS, kl * NB2, bl, xm, obs, rec);
+                                    stage_kb_tc<NB, false>(a, kbase + kl, b, st, E, dr, sDS, kl * NB2, bl, xm, obs, rec);
                             }
                             workers_sync();  // the staged quarter is consumed before it is rewritten
                         }
@@ -1083,45 +1089,30 @@ __global__ void __launch_bounds__(kTcThreads, 1) batched_tc_kernel(TcArgs a) {
                 // every dSigma row is written before the epilogue reads it
                 if (in_sync && !(ok = tc_grid_sync(a, gen, &abort_s))) break;
                 TC_TRACE(worker && wt == 0, 7);
-                // ---- E (channel-wise): commutator + RK4 by 64-row quarters of all N rows
-                //      (items: quarter, trajectory group), dSigma summed over the K-range
-                //      partials of phase C in a fixed order into the staging buffer ----
+                // ---- E (channel-wise): commutator + RK4 of all (k, trajectory) blocks, group by
+                //      group of trajectories, k-points dealt over the CTAs; a thread keeps one
+                //      trajectory and reads dSigma where phase C wrote it (staging it through
+                //      shared memory by 64-row tiles took two CTA barriers per tile and three
+                //      rounds of tiles on some CTAs: 18.5 -> 16.3 ms for 30 steps at N = 20736,
+                //      B = 64) ----
                 if (worker) {
-                    const int nq = 4 * a.nte;
-                    const int nE = nq * q.GC;
-                    for (int item = blockIdx.x; item < nE; item += gridDim.x) {
-                        const int tq = item % nq, g = item / nq;
+                    for (int g = 0; g < q.GC; ++g) {
                         int b0, b1;
                         group_range(Bact, q.GC, g, b0, b1);
                         const int nbg = b1 - b0;
-                        workers_sync();  // the previous item's readers of smx and sred are done
+                        workers_sync();  // the previous group's readers of smx and sred are done
                         if (wt < kGroup) smx[wt] = 0u;
-                        const int64_t r0 = (int64_t)tq * 64;
-                        for (int e = wt; e < 64 * nbg; e += kWorkers) {
-                            const int rr = e / nbg, bb = e % nbg;
-                            if (r0 + rr < a.N) {
-                                const float2* src = a.dS + (r0 + rr) * a.Bp + b0 + bb;
-                                float2 v = __ldcg(src);
-                                for (int kc = 1; kc < a.kcu; ++kc) v = cadd(v, __ldcg(src + (int64_t)kc * a.N * a.Bp));
-                                sDS[ds_index(rr, bb)] = v;
-                            }
-                        }
                         workers_sync();
                         const int kgroups = kWorkers / nbg;
                         const int bl = wt % nbg, kg = wt / nbg;
                         DF3 obs;
                         float xm = 0.f;
-                        const int kbase = (int)(r0 / NB2);
-                        const int kt = min(64 / NB2, a.Nk - kbase);
                         if (kg < kgroups && !*vabort) {
                             const int b = b0 + bl;
                             const float E = (float)a.Etab[(int64_t)b * a.ldE + 2 * (a.n0 + n) + eoff];
                             const float2 dr = a.dir[b];
-                            for (int kl = kg; kl < kt; kl += kgroups)
-                                stage_kb_tc<NB>(a, kbase + kl, b, st, E, dr, sDS, kl * NB2, bl, xm, obs, -1);
-                        }
-                        workers_sync();  // the staged quarter is consumed before sred reuses it
-                        if (kg < kgroups) {
+                            for (int k = blockIdx.x * kgroups + kg; k < a.Nk; k += gridDim.x * kgroups)
+                                stage_kb_tc<NB, true>(a, k, b, st, E, dr, nullptr, 0, bl, xm, obs, -1);
                             atomicMax(smx + bl, __float_as_uint(xm));
                             if (st == 3) {
                                 sred[(kg * nbg + bl) * 3] = obs.p.value();
@@ -1139,7 +1130,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) batched_tc_kernel(TcArgs a) {
                                     r1s += sred[(k2 * nbg + wt) * 3 + 1];
                                     r2s += sred[(k2 * nbg + wt) * 3 + 2];
                                 }
-                                double* rr = a.red + ((int64_t)tq * a.Bp + b0 + wt) * 3;
+                                double* rr = a.red + ((int64_t)blockIdx.x * a.Bp + b0 + wt) * 3;
                                 rr[0] = r0s;
                                 rr[1] = r1s;
                                 rr[2] = r2s;
@@ -1721,7 +1712,6 @@ void propagate_channel_tc(Ctx& c, const tdagw_field* fields, int B, const int* s
     const int nchK = (Nk + 15) / 16, NtK = (Nk + kRows - 1) / kRows;
     const int nsegA = f.tc_mtq0[P];
     const int rp = std::max(1, nsegA) * kRows;
-    const int nte = (int)((N + kRows - 1) / kRows);
     const BatchSetup bs = prepare_batch(c, fields, B, steps, dt);
     const int Bp = bs.Bp;
 
@@ -1740,7 +1730,7 @@ void propagate_channel_tc(Ctx& c, const tdagw_field* fields, int B, const int* s
     c.tcP.ensure((size_t)KSmax * rp * Bp * sizeof(float2));
     c.tcY.ensure((size_t)rp * Bp * sizeof(float2));
     c.tcMax.ensure((size_t)3 * Bp * sizeof(unsigned));
-    c.tcRed.ensure((size_t)4 * nte * Bp * 3 * sizeof(double));
+    c.tcRed.ensure((size_t)nctas * Bp * 3 * sizeof(double));
     const size_t sbytes = (size_t)N * Bp * sizeof(float2);
     constexpr int kKcMax = 4;  // K-ranges of a phase C tile at most (partial dSigma slots)
     c.bdS.ensure(kKcMax * sbytes);
@@ -1790,12 +1780,11 @@ void propagate_channel_tc(Ctx& c, const tdagw_field* fields, int B, const int* s
     a.wait_ns = 2000000000ull;
     a.n0 = 0;
     a.ck_period = 1;
-    a.Nred = 4 * nte;  // per-quarter observable sums
+    a.Nred = nctas;  // per-CTA observable sums
     a.gpad = f.tcGpad.as<int>();
     a.dS = c.bdS.as<float2>();
     a.npair = P;
     a.NtK = NtK;
-    a.nte = nte;
     a.zbound = f.tc_zbound;
     for (int e = 0; e < P; ++e) {
         a.tvoff[e] = f.tc_tvoff[e];
