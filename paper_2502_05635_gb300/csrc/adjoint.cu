@@ -238,15 +238,16 @@ __device__ __noinline__ void phase_dense_adj() {
                           khm + ra * m.Bp + sh.b0, m.Bp, false, nullptr, nullptr);
 }
 
-// dJ/dE at this stage's sample: sum of the row-group partials, one warp per trajectory, fixed
-// order
+// dJ/dE at this stage's sample: sum of the row-group partials in a fixed order, the group's
+// trajectories dealt to the last warps of its CTAs (one CTA alone took 6 us before the barrier)
 __device__ __noinline__ void phase_gradient() {
     AdjShared& as = adj_shared();
     const AdjArgs& a = as.a;
     const BatchArgs& m = as.bs.a;
     const StepShared& sh = as.bs.s;
     const int tid = threadIdx.x, nl = as.bs.n >> 2, s = as.bs.n & 3, eoff = s == 0 ? 0 : (s == 3 ? 2 : 1);
-    for (int b = sh.b0 + (tid >> 5); b < sh.b0 + sh.nb; b += kBThreads / 32) {
+    if ((tid >> 5) != kBThreads / 32 - 1) return;
+    for (int b = sh.b0 + sh.rg; b < sh.b0 + sh.nb; b += sh.Rg) {
         double eb = 0.0;
         for (int g2 = tid & 31; g2 < sh.Rg; g2 += 32) eb += __ldcg(a.red2 + ((int64_t)g2 * m.Bp + b) * 4 + s);
 #pragma unroll
@@ -328,13 +329,13 @@ __global__ void __launch_bounds__(kBThreads, 1) adjoint_kernel(AdjArgs a) {
         if (m.mode == TDAGW_LOWRANK) {
             phase_uhm();
             if (!bgrid_sync(m, bs)) return;
-            if (sh.rg == 0) phase_gradient();
+            phase_gradient();
             phase_sy_adj();
             if (!bgrid_sync(m, bs)) return;
             phase_vy<NB>();
         } else {
             if (!bgrid_sync(m, bs)) return;
-            if (sh.rg == 0) phase_gradient();
+            phase_gradient();
             phase_dense_adj<NB>();
             // all rows of mm are read before the next stage rewrites them
             if (!bgrid_sync(m, bs)) return;

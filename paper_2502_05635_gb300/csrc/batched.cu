@@ -278,6 +278,7 @@ __global__ void __launch_bounds__(kBThreads, 1) batched_kernel(BatchArgs a) {
     if (tid == 0) {
         bs.abort_s = 0;
         bs.gen = 0;
+        bs.n = 0;
         sh.Bact = -1;
     }
     copy_args(bs.a, a);
@@ -285,12 +286,14 @@ __global__ void __launch_bounds__(kBThreads, 1) batched_kernel(BatchArgs a) {
     // observables of step n - 1's end (row n), from the split of that step
     auto last_observables = [&](int n) {
         const StepPlan pp = step_plan(a.act[a.n0 + n - 1], gridDim.x, a.Nk);
-        if (blockIdx.x % pp.Rg == 0 && blockIdx.x / pp.Rg < (unsigned)pp.Tg)
-            reduce_observables_row(a, n, pp, blockIdx.x / pp.Rg);
+        if (blockIdx.x / pp.Rg < (unsigned)pp.Tg)
+            reduce_observables_row(a, n, pp, blockIdx.x / pp.Rg, blockIdx.x % pp.Rg);
     };
-    for (int gs = 0; gs < 4 * a.Tmax; ++gs) {  // one counter for step and stage: it lives across the calls
-        const int n = gs >> 2;
-        const int st = gs & 3;
+    // stage counter (4 step + stage), read from shared memory so that no register holds it
+    // across the calls
+    volatile int& gs = bs.n;
+    while (gs < 4 * a.Tmax) {
+        const int n = gs >> 2, st = gs & 3;
         if (st == 0) {
             // this step's block of the split
             if (tid == 0) {
@@ -315,12 +318,12 @@ __global__ void __launch_bounds__(kBThreads, 1) batched_kernel(BatchArgs a) {
                 a.ckC[slot + off] = __ldcg(a.Ccomp + off);
             }
         }
-        // observables of step n-1 (written by the CTAs of that step's row group 0)
+        // observables of step n-1
         if (st == 0 && n > 0 && a.mode == TDAGW_FULL) last_observables(n);
         if (a.mode != TDAGW_FULL) {
             phase_vhx<NB, CH>();
             if (!bgrid_sync(a, bs)) return;
-            if (st == 0 && n > 0) last_observables(n);
+            if ((gs & 3) == 0 && gs > 0) last_observables(gs >> 2);
             phase_sy<NB, CH>();
             if (!bgrid_sync(a, bs)) return;
             phase_uy<NB, CH>();
@@ -334,6 +337,8 @@ __global__ void __launch_bounds__(kBThreads, 1) batched_kernel(BatchArgs a) {
         }
         __syncthreads();
         epilogue<NB>(a, bs, gs);
+        if (tid == 0) gs = gs + 1;
+        __syncthreads();
     }
     // observables of the last step
     if (a.Tmax > 0 && bgrid_sync(a, bs)) last_observables(a.Tmax);

@@ -212,10 +212,10 @@ template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.as
 // tiles with the reduction split over up to 8 slices, whose partial tiles are added in a
 // fixed order through the idle staging memory: results are deterministic.  acc adds to out.
 // Measured alone on 152 SMs, 32 columns: 52 TFLOP/s at 512 x 512, 42 at 256 x 121 and
-// 121 x 256, 31 at 36 x 512 (64 is the FMA ceiling above).  With step_plan, against the
-// former 4 x 4 single-buffered tile and fixed split: the field sweep 55.5 -> 35.5 ms (256
+// 121 x 256, 34 at 36 x 512 (64 is the FMA ceiling above).  With step_plan, against the
+// former 4 x 4 single-buffered tile and fixed split: the field sweep 55.5 -> 34.0 ms (256
 // uneven trajectories of 20-160 steps, N = 2304, rank 256), checkpointed forward and gradients
-// of 32 trajectories 56.6 -> 35.1 ms (49 steps, N = 5184, rank 512).
+// of 32 trajectories 56.6 -> 31.5 ms (49 steps, N = 5184, rank 512).
 template <bool TRANS, int TM, int LKS>
 __device__ __noinline__ void block_gemm_tile() {
     BatchShared& bs = batch_shared();
@@ -229,12 +229,13 @@ __device__ __noinline__ void block_gemm_tile() {
     constexpr int tyc = ng / 8;                // row groups
     constexpr int Mt = TM * tyc;               // rows per pass
     constexpr int ldq = Mt + 4;                // complex per staged A row
-    constexpr int TP = TM / 2;                 // row pairs per thread: rows 2 ty + 2 tyc u, + 1
+    // rows of a thread: TM / 2 pairs 2 ty + 2 tyc u, + 1, and one more when TM is odd
+    constexpr int TP = TM / 2;
     static_assert(ks * kDepth * ldq * 2 <= kStageA && ks * kDepth * kTileB * 2 <= kStageB, "stage size");
-    static_assert(TM % 2 == 0, "row pairs");
     const int tid = threadIdx.x;
     const int slice = tid / ng, tl = tid % ng;
     const int tx = tl % 8, ty = tl / 8;
+    auto row_of = [&](int u) { return u < 2 * TP ? 2 * ty + 2 * tyc * (u >> 1) + (u & 1) : 2 * tyc * TP + ty; };
     for (int m0 = 0; m0 < M; m0 += Mt) {
         const int mrows = min(Mt, M - m0);
         float2 c[TM][4];
@@ -322,12 +323,16 @@ __device__ __noinline__ void block_gemm_tile() {
             sA += slice * kDepth * ldq;
             const int kc = depth(ch);
             auto fma_row = [&](int q) {
-                float4 av[TP], bv[2];
+                float4 av[TP + (TM & 1)], bv[2];
                 // columns 2 tx, 2 tx + 1, 16 + 2 tx, 17 + 2 tx
                 bv[0] = *reinterpret_cast<const float4*>(sB + q * kTileB + 2 * tx);
                 bv[1] = *reinterpret_cast<const float4*>(sB + q * kTileB + 16 + 2 * tx);
 #pragma unroll
                 for (int u = 0; u < TP; ++u) av[u] = *reinterpret_cast<const float4*>(sA + q * ldq + 2 * ty + 2 * tyc * u);
+                if (TM & 1) {
+                    const float2 z = sA[q * ldq + 2 * tyc * TP + ty];
+                    av[TM / 2] = make_float4(z.x, z.y, 0.f, 0.f);
+                }
 #pragma unroll
                 for (int u = 0; u < TM; ++u) {
                     const float4 a4 = av[u / 2];
@@ -366,7 +371,7 @@ __device__ __noinline__ void block_gemm_tile() {
             for (int u = 0; u < TM; ++u)
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
-                    const int b = (v >> 1) * 16 + 2 * tx + (v & 1), m = 2 * ty + 2 * tyc * (u >> 1) + (u & 1);
+                    const int b = (v >> 1) * 16 + 2 * tx + (v & 1), m = row_of(u);
                     if (b < nb && m < mrows) finish(m0 + m, b, c[u][v]);
                 }
             __syncthreads();  // the staging memory is reused
@@ -377,8 +382,7 @@ __device__ __noinline__ void block_gemm_tile() {
             for (int u = 0; u < TM; ++u)
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
-                    *reinterpret_cast<float4*>(red + (slice * Mt + 2 * ty + 2 * tyc * (u >> 1) + (u & 1)) * kTileB +
-                                               16 * h + 2 * tx) =
+                    *reinterpret_cast<float4*>(red + (slice * Mt + row_of(u)) * kTileB + 16 * h + 2 * tx) =
                         make_float4(c[u][2 * h].x, c[u][2 * h].y, c[u][2 * h + 1].x, c[u][2 * h + 1].y);
             __syncthreads();
             for (int e = tid; e < mrows * kTileB; e += kBThreads) {
@@ -433,7 +437,8 @@ static __device__ __forceinline__ void block_gemm(const float2* __restrict__ A, 
         if (M > 128) block_gemm_tile<TRANS, 8, 1>();
         else if (M > 64) block_gemm_tile<TRANS, 8, 2>();
         else if (M > 48) block_gemm_tile<TRANS, 8, 3>();
-        else if (M > 32) block_gemm_tile<TRANS, 6, 3>();
+        else if (M > 40) block_gemm_tile<TRANS, 6, 3>();
+        else if (M > 32) block_gemm_tile<TRANS, 5, 3>();
         else if (M > 16) block_gemm_tile<TRANS, 4, 3>();
         else block_gemm_tile<TRANS, 2, 3>();
     }
@@ -492,12 +497,15 @@ static __device__ void reduce_partials(const float2* __restrict__ P, int64_t pst
 }
 
 // Observables of step n (rows of a.obs) of the trajectories of group tg at that step from the
-// row groups' partials: one warp per trajectory, lanes over the row groups, fixed order.
-static __device__ void reduce_observables_row(const BatchArgs& a, int n, const StepPlan& pl, int tg) {
+// row groups' partials: one warp per trajectory, lanes over the row groups, fixed order.  The
+// trajectories are dealt to the last warps of the group's CTAs (rg of Rg): one CTA alone held
+// up the next barrier by 4 us.
+static __device__ void reduce_observables_row(const BatchArgs& a, int n, const StepPlan& pl, int tg, int rg) {
+    if ((threadIdx.x >> 5) != kBThreads / 32 - 1) return;
     int p0, p1;
     group_range(a.act[a.n0 + n - 1], pl.Tg, tg, p0, p1);
     const int lane = threadIdx.x & 31;
-    for (int b = p0 + (int)(threadIdx.x >> 5); b < p1; b += kBThreads / 32) {
+    for (int b = p0 + rg; b < p1; b += pl.Rg) {
         double s0 = 0, s1 = 0, s2 = 0;
         for (int g = lane; g < pl.Rg; g += 32) {
             const double* rr = a.red + ((int64_t)g * a.Bp + b) * 3;
