@@ -10,14 +10,20 @@
 //             (G x rank, fixed order), scales by S and multiplies its rows of U
 //   then the commutator, the RK4 stage update and the observables in registers.
 //
-// Bound by the one grid barrier per stage and the L2 round trips around it.  The stage-wise
+// The smallest models fit in one cluster of up to 16 CTAs: the exchange then goes through
+// distributed shared memory (every CTA writes its part into the others') and the cluster's
+// hardware barrier instead of L2 and a counter.
+//
+// Bound by the one barrier per stage and the exchange around it.  The stage-wise
 // path of the dense kernel takes two launches per stage; the streaming low-rank kernel
 // (lr_persistent.cu) two barriers, and its state goes through L2.  The exchange buffers
 // alternate by stage parity: a CTA writes the next stage's while a slower one still reads.
 // Waits are bounded as in the other persistent kernels.
 //
-// Measured per stage: dense, N = 576 6.1 -> 3.6 us (stage-wise before); low rank, N = 2116,
-// rank 235 9.3 -> 5.7 us (streaming kernel before).
+// Measured per stage: dense, N = 576 6.1 us (stage-wise) -> 3.6 (grid) -> 2.7 (cluster); low
+// rank, N = 2116, rank 235 9.3 us (streaming kernel) -> 5.6 (grid).
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 
@@ -30,7 +36,9 @@ namespace tdagw {
 namespace {
 
 using namespace persist;
+namespace cg = cooperative_groups;
 
+constexpr int kClMax = 16;  // CTAs of a cluster (above 8: opt-in)
 constexpr int kRThreads = 512, kRWarps = kRThreads / 32;
 constexpr size_t kRSmem = 224 * 1024;  // dynamic shared memory at most
 
@@ -88,28 +96,40 @@ __device__ __forceinline__ void row_pass(const float2* A, int ld, int nrows, int
                 acc[w] = cfma(make_float2(a.z, a.w), make_float2(xv.z, xv.w), acc[w]);
             }
         }
+        // sums over the lanes: W rows are halved between the lane halves first
+        int o = 16;
 #pragma unroll
-        for (int w = 0; w < W; ++w) {
+        for (int h = W; h > 1; h >>= 1, o >>= 1) {
+            const bool up = lane & o;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc[w] = cadd(acc[w], shfl_xor(acc[w], o));
-            if (lane == 0 && r0 + w < nrows) dots[part * rows_max + r0 + w] = acc[w];
+            for (int q = 0; q < h / 2; ++q) {
+                const float2 keep = up ? acc[q + h / 2] : acc[q], send = up ? acc[q] : acc[q + h / 2];
+                acc[q] = cadd(keep, shfl_xor(send, o));
+            }
         }
+        float2 s = acc[0];
+#pragma unroll
+        for (; o > 0; o >>= 1) s = cadd(s, shfl_xor(s, o));
+        const int row = r0 + lane / (32 / W);
+        if (lane % (32 / W) == 0 && row < nrows) dots[part * rows_max + row] = s;
     }
 }
 
-template <int NB, bool LR>
+// CL: the grid is one cluster
+template <int NB, bool LR, bool CL>
 __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(ResArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int P = NB * NB;
     const int G = gridDim.x, cta = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int ka = (int)((int64_t)cta * a.Nk / G), kb = (int)((int64_t)(cta + 1) * a.Nk / G);
     const int ra = ka * P, nrows = (kb - ka) * P, ld = (int)a.ld;
-    const int nv = LR ? ld : a.N + (a.N & 1);  // length of the exchanged vector in shared memory
+    const int nv = LR ? ld : a.N;  // length of the exchanged vector (N is even: Nb^2 a multiple of 4)
 
     float2* As = reinterpret_cast<float2*>(smem);               // rows_max x ld
     float2* Vs = As + (int64_t)a.rows_max * ld;                 // low rank: rows_max x ld
-    float2* vec = Vs + (LR ? (int64_t)a.rows_max * ld : 0);     // S o y, or X
-    float2* xs = vec + nv;                                      // own stage input (low rank)
+    float2* vec = Vs + (LR ? (int64_t)a.rows_max * ld : 0);     // S o y, or X (cluster: two X, by parity)
+    float2* pcl = vec + (CL && !LR ? 2 : 1) * nv;               // cluster, low rank: 2 x G partial vectors
+    float2* xs = pcl + (CL && LR ? 2 * (int64_t)G * ld : 0);    // own stage input (low rank)
     float2* dots = xs + a.rows_max;                             // parts x rows_max
     float2* sub = dots + kRWarps * a.rows_max;                  // low rank: 2 x kRThreads partial sums
     __shared__ float wf[6 * kRWarps];
@@ -119,7 +139,7 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(ResArgs a) {
     if (tid == 0) abort_flag = 0;
     load_rows(As, a.A + (int64_t)ra * ld, (int64_t)nrows * ld);
     if (LR) load_rows(Vs, a.V + (int64_t)ra * ld, (int64_t)nrows * ld);
-    if (!LR && tid == 0 && (a.N & 1)) vec[a.N] = make_float2(0.f, 0.f);
+    __shared__ double cobs[2][kClMax][3];  // cluster: the CTAs' observables, in the last CTA
 
     // this thread's pair element (nrows <= kRThreads)
     const bool act = tid < nrows;
@@ -157,6 +177,7 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(ResArgs a) {
             wf[6 * warp + 5] = ob.o.lo;
         }
     };
+    int opar = 0;
     auto publish_observables = [&]() {
         if (tid >= 3) return;
         DF s;
@@ -166,12 +187,25 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(ResArgs a) {
             t.lo = wf[6 * w + 2 * tid + 1];
             s.add(t);
         }
-        __stcg(a.red + 3 * cta + tid, s.value());
+        // (alternating by step in the cluster: the last CTA may still read the previous one)
+        if (CL) cg::this_cluster().map_shared_rank(&cobs[opar][cta][tid], G - 1)[0] = s.value();
+        else __stcg(a.red + 3 * cta + tid, s.value());
+    };
+    // row `row` of the observables from the CTAs' sums (one warp of the last CTA, fixed order)
+    auto write_observables = [&](int64_t row) {
+        if (!CL) {
+            reduce_obs_row(a.red, G, 1.0 / (double)a.Nk, a.obs + 3 * row, lane);
+        } else if (lane < 3) {
+            double s = 0.0;
+            for (int c = 0; c < G; ++c) s += cobs[opar][c][lane];
+            a.obs[3 * row + lane] = s * (1.0 / (double)a.Nk);
+        }
     };
     if (act) xs[tid] = X;
     warp_observables();  // row 0, by the same sums as every other row (a resumed run repeats it)
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
+    if (CL) cg::this_cluster().sync();  // every CTA runs: its shared memory may be written
     publish_observables();
 
     // column parts of the row pass: as many as the groups of four rows leave warps for
@@ -194,7 +228,6 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(ResArgs a) {
                 }
                 s = make_float4(y0.x, y0.y, y1.x, y1.y);
             }
-            float2* mine = a.xch + ((int64_t)par * G + cta) * ld;
             if (nsub > 1) {
                 if (sb < nsub) reinterpret_cast<float4*>(sub)[tid] = s;
                 __syncthreads();
@@ -207,23 +240,33 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(ResArgs a) {
                         s.w += t.w;
                     }
             }
-            if (tid < ncp) __stcg(reinterpret_cast<float4*>(mine + 2 * tid), s);
-        } else {
-            if (act) __stcg(a.xch + (int64_t)par * a.N + i, X);
+            const int64_t off = ((int64_t)par * G + cta) * ld + 2 * tid;
+            if (tid < ncp) {
+                if (CL)
+                    for (int c = 0; c < G; ++c)
+                        *reinterpret_cast<float4*>(cg::this_cluster().map_shared_rank(pcl + off, c)) = s;
+                else
+                    __stcg(reinterpret_cast<float4*>(a.xch + off), s);
+            }
+        } else if (act) {
+            if (CL)
+                for (int c = 0; c < G; ++c) *cg::this_cluster().map_shared_rank(vec + (int64_t)par * nv + i, c) = X;
+            else
+                __stcg(a.xch + (int64_t)par * a.N + i, X);
         }
-        if (!grid_sync<kRThreads>(a.bar_count, a.err, a.extra_arrivals, a.wait_ns, lgen, abort_s)) return;
+        if (CL) cg::this_cluster().sync();
+        else if (!grid_sync<kRThreads>(a.bar_count, a.err, a.extra_arrivals, a.wait_ns, lgen, abort_s)) return;
         // observables after the previous step, or of the start (published before this barrier)
-        if (st == 0 && cta == G - 1 && warp == kRWarps - 1)
-            reduce_obs_row(a.red, G, 1.0 / (double)a.Nk, a.obs + 3 * (int64_t)n, lane);
+        if (st == 0 && cta == G - 1 && warp == kRWarps - 1) write_observables(n);
         if (LR) {
             // ---- S o sum of all partial vectors: thread = (column pair, subset of the CTAs)
             const int ncp = ld / 2, nsub = kRThreads / ncp, cp = tid % ncp, sb = tid / ncp;
             float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-            const float4* src = reinterpret_cast<const float4*>(a.xch + (int64_t)par * G * ld) + cp;
+            const float4* src = reinterpret_cast<const float4*>((CL ? pcl : a.xch) + (int64_t)par * G * ld) + cp;
             if (sb < nsub) {
 #pragma unroll 8
                 for (int c = sb; c < G; c += nsub) {
-                    const float4 t = __ldcg(src + (int64_t)c * ncp);
+                    const float4 t = CL ? src[(int64_t)c * ncp] : __ldcg(src + (int64_t)c * ncp);
                     s.x += t.x;
                     s.y += t.y;
                     s.z += t.z;
@@ -243,13 +286,13 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(ResArgs a) {
                 const float s0 = a.S[2 * tid], s1 = 2 * tid + 1 < a.r ? a.S[2 * tid + 1] : 0.f;
                 reinterpret_cast<float4*>(vec)[tid] = make_float4(s.x * s0, s.y * s0, s.z * s1, s.w * s1);
             }
-        } else {
-            for (int e = 2 * tid; e < a.N; e += 2 * kRThreads)  // N is even (Nb^2 a multiple of 4)
+        } else if (!CL) {
+            for (int e = 2 * tid; e < a.N; e += 2 * kRThreads)
                 *reinterpret_cast<float4*>(vec + e) =
                     __ldcg(reinterpret_cast<const float4*>(a.xch + (int64_t)par * a.N + e));
         }
-        __syncthreads();
-        row_pass<4>(As, ld, nrows, a.rows_max, parts, vec, dots, warp, lane);
+        if (LR || !CL) __syncthreads();
+        row_pass<4>(As, ld, nrows, a.rows_max, parts, vec + (CL && !LR ? (int64_t)par * nv : 0), dots, warp, lane);
         __syncthreads();
         // ---- commutator and RK4 stage update (the arithmetic of stage_element)
         float2 dS = act ? dots[tid] : zero;
@@ -287,17 +330,20 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(ResArgs a) {
         }
         if (LR && act) xs[tid] = X;
         __syncthreads();
-        if (st == 3) publish_observables();
+        if (st == 3) {
+            opar ^= 1;
+            publish_observables();
+        }
     }
     if (act) {
         a.X[i] = X;
         a.Ssum[i] = Ss;
         a.Ccomp[i] = Cc;
     }
-    // observables of the last step
-    if (a.T > 0 && grid_sync<kRThreads>(a.bar_count, a.err, a.extra_arrivals, a.wait_ns, lgen, abort_s) &&
-        cta == G - 1 && warp == 0)
-        reduce_obs_row(a.red, G, 1.0 / (double)a.Nk, a.obs + 3 * (int64_t)a.T, lane);
+    // observables of the last step (cluster: no CTA leaves while another writes its memory)
+    if (CL) cg::this_cluster().sync();
+    else if (!grid_sync<kRThreads>(a.bar_count, a.err, a.extra_arrivals, a.wait_ns, lgen, abort_s)) return;
+    if (cta == G - 1 && warp == 0) write_observables(a.T);
 }
 
 }  // namespace
@@ -318,20 +364,59 @@ bool launch_resident(Ctx& c, int mode, int T, double dt, double dirx, double dir
     TDAGW_CUDA(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     TDAGW_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
     if (!coop) return false;
-    auto smem_for = [&](int rows) {
-        return (size_t)((lr ? 2 : 1) * (int64_t)rows * ld + (lr ? ld : N) + rows + (int64_t)kRWarps * rows +
+    const size_t cap = std::min(kRSmem, (size_t)smem_max - 4096);
+    auto smem_for = [&](int rows, int gcl) {  // gcl: CTAs of the cluster, 0: grid
+        const int64_t vecs = lr ? ld + 2 * gcl * ld : (gcl ? 2 : 1) * N;
+        return (size_t)((lr ? 2 : 1) * (int64_t)rows * ld + vecs + rows + (int64_t)kRWarps * rows +
                         (lr ? 2 * kRThreads : 0)) * sizeof(float2);
     };
-    const size_t cap = std::min(kRSmem, (size_t)smem_max - 2048);
-    // k-points per CTA: low rank about sqrt(N) CTAs (a CTA reads its share of the factors and
-    // one partial vector per CTA: 2 N / G + G rows, least at G = sqrt(N)); dense eight rows
-    const int Gw = lr ? (int)std::lround(std::sqrt((double)N)) : (int)((N + 7) / 8);
-    int G = std::max(1, std::min({Gw, nsm, h.Nk}));
     auto rows_of = [&](int g) { return (h.Nk + g - 1) / g * P; };
-    while (G < std::min(nsm, h.Nk) && (rows_of(G) > kRThreads || smem_for(rows_of(G)) > cap)) ++G;
+    auto kernel = [&](bool cl) -> const void* {
+        if (h.Nb == 2) {
+            if (lr) return cl ? (const void*)resident_kernel<2, true, true> : (const void*)resident_kernel<2, true, false>;
+            return cl ? (const void*)resident_kernel<2, false, true> : (const void*)resident_kernel<2, false, false>;
+        }
+        if (lr) return cl ? (const void*)resident_kernel<4, true, true> : (const void*)resident_kernel<4, true, false>;
+        return cl ? (const void*)resident_kernel<4, false, true> : (const void*)resident_kernel<4, false, false>;
+    };
+    // one cluster when the kernel fits in it (and the device has room for such a cluster); the
+    // bounded waits of the timeout test are those of the grid
+    int G = 1;
+    while (2 * G <= std::min(kClMax, h.Nk)) G *= 2;
+    bool cl = !test_timeout && rows_of(G) <= kRThreads && smem_for(rows_of(G), G) <= cap;
+    cudaLaunchAttribute attr{};
+    cudaLaunchConfig_t cfg{};
+    if (cl) {
+        const void* fn = kernel(true);
+        const size_t sm = smem_for(rows_of(G), G);
+        TDAGW_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        TDAGW_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = (unsigned)G;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.gridDim = dim3(G);
+        cfg.blockDim = dim3(kRThreads);
+        cfg.dynamicSmemBytes = sm;
+        cfg.stream = s;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        int ncl = 0;
+        if (cudaOccupancyMaxActiveClusters(&ncl, fn, &cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            ncl = 0;
+        }
+        cl = ncl >= 1;
+    }
+    if (!cl) {
+        // k-points per CTA: low rank about sqrt(N) CTAs (a CTA reads its share of the factors
+        // and one partial vector per CTA: 2 N / G + G rows, least at G = sqrt(N)); dense eight rows
+        const int Gw = lr ? (int)std::lround(std::sqrt((double)N)) : (int)((N + 7) / 8);
+        G = std::max(1, std::min({Gw, nsm, h.Nk}));
+        while (G < std::min(nsm, h.Nk) && (rows_of(G) > kRThreads || smem_for(rows_of(G), 0) > cap)) ++G;
+        if (rows_of(G) > kRThreads || smem_for(rows_of(G), 0) > cap) return false;
+        if (lr && (int64_t)G * ld * 8 > 160 * 1024) return false;
+    }
     const int rows_max = rows_of(G);
-    if (rows_max > kRThreads || smem_for(rows_max) > cap) return false;
-    if (lr && (int64_t)G * ld * 8 > 160 * 1024) return false;
 
     ResArgs a{};
     a.A = lr ? c.U.as<float2>() : c.K.as<float2>();
@@ -370,14 +455,17 @@ bool launch_resident(Ctx& c, int mode, int T, double dt, double dirx, double dir
     a.extra_arrivals = test_timeout ? 1 : 0;
     a.wait_ns = test_timeout ? 20000000ull : 2000000000ull;
     void* args[] = {&a};
-    const void* fn = h.Nb == 2 ? (lr ? (const void*)resident_kernel<2, true> : (const void*)resident_kernel<2, false>)
-                               : (lr ? (const void*)resident_kernel<4, true> : (const void*)resident_kernel<4, false>);
-    const size_t smem = smem_for(rows_max);
-    TDAGW_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int per_sm = 0;
-    TDAGW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kRThreads, smem));
-    if (per_sm < 1) return false;
-    TDAGW_CUDA(cudaLaunchCooperativeKernel(fn, dim3(G), dim3(kRThreads), args, smem, s));
+    const void* fn = kernel(cl);
+    if (cl) {
+        TDAGW_CUDA(cudaLaunchKernelExC(&cfg, fn, args));
+    } else {
+        const size_t smem = smem_for(rows_max, 0);
+        TDAGW_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        int per_sm = 0;
+        TDAGW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kRThreads, smem));
+        if (per_sm < 1) return false;
+        TDAGW_CUDA(cudaLaunchCooperativeKernel(fn, dim3(G), dim3(kRThreads), args, smem, s));
+    }
     c.persistent_launched = true;
     return true;
 }

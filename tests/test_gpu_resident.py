@@ -46,13 +46,14 @@ def _run(p, mode, apply, install=None, T=24):
     np.testing.assert_allclose(b[0], got[9], rtol=1e-10, atol=1e-15)
 
 
-@pytest.mark.parametrize("L,nc", [(8, 1), (9, 1), (5, 2), (12, 1), (21, 1), (22, 1), (11, 2), (23, 1)])
+@pytest.mark.parametrize("L,nc", [(8, 1), (9, 1), (5, 2), (12, 1), (13, 1), (7, 2), (21, 1), (22, 1), (11, 2), (23, 1)])
 def test_dense(L, nc):
     _run(wl.small_model(L, nc), tg.FULL, lambda m: (lambda K: (lambda v: K @ v))(ok.dense_kernel(m)))
 
 
 @pytest.mark.parametrize("L,nc,rank", [(2, 1, 1), (3, 2, 2), (9, 1, 7), (12, 1, 29), (23, 1, 235), (24, 1, 256),
-                                       (24, 1, 400), (11, 2, 129), (13, 2, 64), (5, 1, 100), (30, 1, 511)])
+                                       (24, 1, 400), (11, 2, 129), (13, 2, 64), (5, 1, 100), (30, 1, 511),
+                                       (12, 1, 300), (12, 1, 340), (24, 1, 70), (3, 1, 36), (16, 2, 33)])
 def test_lowrank(L, nc, rank):
     p = wl.small_model(L, nc)
     U, S, V, d = wl.random_factors(p.N, rank, seed=rank + L)
