@@ -66,6 +66,8 @@ struct LRArgs {
     int64_t N;
     int Nk, r, ldu, T;
     int rows_per_slot, nslots, slot_bytes, rows_max;
+    int pf_tiles;        // tiles prefetched into L2 once the ring is full of a pass's first ones
+    int upart_len;       // float2 entries of upart
     int u_parts, u_part_w;  // U pass: column parts per row (power of 2) and their width
     int extra_arrivals;  // > 0 only for the timeout test: the barrier can never complete
     unsigned long long wait_ns;
@@ -74,6 +76,9 @@ struct LRArgs {
 #ifndef TDAGW_LR_EVICT_FIRST
 #define TDAGW_LR_EVICT_FIRST 1  // factor rows streamed with an L2 evict-first policy (read once per stage)
 #endif
+__device__ __forceinline__ void l2_prefetch(const void* src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void consumer_sync() { named_sync<kConsumers>(); }
 
 // Grid-wide barrier among the consumer threads of all CTAs (monotonic arrival counter; see
@@ -104,9 +109,10 @@ __global__ void __launch_bounds__(kThreads, 1) lr_persistent_kernel(LRArgs a) {
     unsigned char* ring = smem;
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)ns * a.slot_bytes);
     uint64_t* empty = full + ns;
-    // partial U-pass dot products: rows_max x u_parts (at least ldu entries of room)
+    // partial U-pass dot products: rows_max x u_parts (at least ldu entries of room, and the
+    // V pass's partial sums of its row subsets)
     float2* upart = reinterpret_cast<float2*>(empty + ns);
-    float2* xs = upart + max(ldu, a.rows_max * a.u_parts);
+    float2* xs = upart + a.upart_len;
     double* wred = reinterpret_cast<double*>(xs + a.rows_max);
     volatile int* abort_s = reinterpret_cast<volatile int*>(wred + 3 * kConsumerWarps);
 
@@ -151,6 +157,12 @@ __global__ void __launch_bounds__(kThreads, 1) lr_persistent_kernel(LRArgs a) {
                                          bytes, full + pos.slot);
                             ++issued;
                             pos.advance(1, ns);
+                            // the ring is full of this pass's first tiles, the consumers are at
+                            // the barriers before it: start the next tiles' way from HBM to L2
+                            if (t == ns - 1) {
+                                const int r1 = (t + 1) * rps, r2 = min(nrows, r1 + a.pf_tiles * rps);
+                                if (r2 > r1) l2_prefetch(base + (int64_t)r1 * ldu, (uint32_t)(r2 - r1) * ldu * 8u);
+                            }
                         }
                     }
             if (!ok) {
@@ -174,6 +186,9 @@ __global__ void __launch_bounds__(kThreads, 1) lr_persistent_kernel(LRArgs a) {
         // ------------------------------------------------------------ consumer warps
         const int64_t ea = ra, eb = rb;
         const int jr0 = (int)((int64_t)cta * a.r / G), jr1 = (int)((int64_t)(cta + 1) * a.r / G);
+        // V pass by row subsets: vsub of them (1: all rows, more than 256 column pairs)
+        const int vsub = ldu <= kConsumers ? 2 * kConsumers / ldu : 1;
+        const int vcp = vsub > 1 ? tid % (ldu / 2) : 0, vsb = vsub > 1 ? tid / (ldu / 2) : 0;
         unsigned lgen = 0;
         RingPos pos{0, 0u};
         bool ok = true;
@@ -182,8 +197,11 @@ __global__ void __launch_bounds__(kThreads, 1) lr_persistent_kernel(LRArgs a) {
         for (int n = 0; n < a.T && ok; ++n) {
             for (int st = 0; st < 4 && ok; ++st) {
                 TDAGW_TRACE_POINT(0);
-                // ---- V pass: every warp reads every row; thread owns column pairs
-                //      tid and tid + 512 (ldu <= 2048)
+                // ---- V pass: thread owns column pairs tid and tid + 512 (ldu <= 2048) of every
+                //      row; with at most 256 column pairs, one pair (vcp) of every vsub-th row,
+                //      so that short rows keep all warps busy (up to 512 columns half of them
+                //      and more had no column): N = 20736 rank 512 32.9 -> 29.7 us / stage,
+                //      rank 200 24.5 -> 17.0; N = 9216 rank 350 18.1 -> 15.7
                 float2 acc[4];
 #pragma unroll
                 for (int m = 0; m < 4; ++m) acc[m] = make_float2(0.f, 0.f);
@@ -191,7 +209,14 @@ __global__ void __launch_bounds__(kThreads, 1) lr_persistent_kernel(LRArgs a) {
                     if (!warp_wait_full(full, pos, abort_s, a.wait_ns, lane)) break;
                     const float2* tile = reinterpret_cast<const float2*>(ring + (size_t)pos.slot * a.slot_bytes);
                     const int r0 = t * rps, nr = min(rps, nrows - r0);
-                    for (int rr = 0; rr < nr; ++rr) {
+                    if (vsub > 1) {
+                        for (int rr = vsb; rr < nr; rr += vsub) {
+                            const float2 xi = xs[r0 + rr];
+                            const float4 v = *reinterpret_cast<const float4*>(tile + (size_t)rr * ldu + 2 * vcp);
+                            acc[0] = cfmac(make_float2(v.x, v.y), xi, acc[0]);
+                            acc[1] = cfmac(make_float2(v.z, v.w), xi, acc[1]);
+                        }
+                    } else for (int rr = 0; rr < nr; ++rr) {
                         const float2 xi = xs[r0 + rr];
                         const float2* row = tile + (size_t)rr * ldu;
 #pragma unroll
@@ -209,6 +234,18 @@ __global__ void __launch_bounds__(kThreads, 1) lr_persistent_kernel(LRArgs a) {
                     pos.advance(1, ns);
                 }
                 TDAGW_TRACE_POINT(1);
+                if (vsub > 1) {
+                    // the row subsets' sums, added in order (upart is idle until the U pass)
+                    if (vsb < vsub)
+                        reinterpret_cast<float4*>(upart)[tid] = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
+                    consumer_sync();
+                    if (2 * tid < ldu)
+                        for (int u = 1; u < vsub; ++u) {
+                            const float4 t4 = reinterpret_cast<const float4*>(upart)[u * (ldu / 2) + tid];
+                            acc[0] = cadd(acc[0], make_float2(t4.x, t4.y));
+                            acc[1] = cadd(acc[1], make_float2(t4.z, t4.w));
+                        }
+                }
 #pragma unroll
                 for (int m = 0; m < 2; ++m) {
                     const int p = tid + m * kConsumers;
@@ -393,8 +430,8 @@ bool launch_lr_persistent(Ctx& c, int T, double dt, double dirx, double diry, bo
     // U pass: rows per slot x column parts = 16 consumer warps (parts of even width)
     const int u_parts = rps >= kConsumerWarps ? 1 : kConsumerWarps / rps;
     const int u_part_w = ((ldu + u_parts - 1) / u_parts + 1) / 2 * 2;
-    const size_t extras = (size_t)std::max(ldu, rows_max * u_parts) * 8 + (size_t)rows_max * 8 +
-                          3 * kConsumerWarps * 8 + 16;
+    const int upart_len = (std::max({ldu, rows_max * u_parts, ldu <= kConsumers ? 2 * kConsumers : 0}) + 1) / 2 * 2;
+    const size_t extras = (size_t)upart_len * 8 + (size_t)rows_max * 8 + 3 * kConsumerWarps * 8 + 16;
     const size_t avail = (size_t)smem_max - 1024;
     if (avail < extras + 4 * (size_t)slot_bytes) return false;
     const int nslots = (int)std::min<size_t>(64, (avail - extras) / (slot_bytes + 16));
@@ -449,6 +486,18 @@ bool launch_lr_persistent(Ctx& c, int T, double dt, double dirx, double diry, bo
     a.nslots = nslots;
     a.slot_bytes = slot_bytes;
     a.rows_max = rows_max;
+    a.upart_len = upart_len;
+    // tiles started towards L2 while the ring is full before a pass, only where the factors are
+    // far larger than L2 (else they push out lines of the other pass): at this point the HBM
+    // queue idles until the barriers before the pass are through.  us / stage without and with:
+    // N = 20736, rank 1024 (340 MB) 55.4 -> 53.6 with two tiles (52.9 with four, 54.1 with
+    // eight: of more tiles a part stays in L2 until the next stage, and the traffic test holds
+    // the DRAM reads of a stage to the factors' size), N = 36864 with eight, rank 1024 (604 MB)
+    // 96.8 -> 91.0, rank 2047 187.5 -> 182.3; rank 512 of N = 20736 (170 MB) 33.5 -> 34.5 with six
+    int l2 = 0;
+    TDAGW_CUDA(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
+    const int64_t factor_bytes = 2 * h.N * (int64_t)row_bytes;
+    a.pf_tiles = factor_bytes > 4 * (int64_t)l2 ? 8 : (factor_bytes > 2 * (int64_t)l2 ? 2 : 0);
     a.u_parts = u_parts;
     a.u_part_w = u_part_w;
     a.extra_arrivals = test_timeout ? 1 : 0;
