@@ -58,11 +58,11 @@ enum {
     TDAGW_FLAG_RESET = 1,         /* start from drho = 0 and t = 0 (else continue)          */
     TDAGW_FLAG_NO_GRAPH = 2,      /* launch stage by stage instead of replaying a CUDA graph */
     TDAGW_FLAG_NO_KAHAN = 4,      /* plain (uncompensated) RK4 accumulation                 */
-    TDAGW_FLAG_STAGEWISE = 8,     /* low-rank or channel-wise c64: stage-wise kernels
-                                     instead of the persistent single-launch kernel         */
+    TDAGW_FLAG_STAGEWISE = 8,     /* c64: stage-wise kernels instead of the persistent or
+                                     on-chip single-launch kernel                           */
     TDAGW_FLAG_TEST_TIMEOUT = 16, /* fault-injection hook for tests: the grid barrier of the
-                                     persistent single-trajectory kernels and of the
-                                     batched kernels (no tuning runs then) waits
+                                     low-rank and channel-wise single-launch kernels and of
+                                     the batched kernels (no tuning runs then) waits
                                      for one block that does not exist,
                                      every wait runs out a 20 ms budget and the call ends
                                      with TDAGW_ERR_TIMEOUT at the next synchronising call   */

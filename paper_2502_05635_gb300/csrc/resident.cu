@@ -356,8 +356,9 @@ bool launch_resident(Ctx& c, int mode, int T, double dt, double dirx, double dir
     if (c.dtype != TDAGW_C64 || (lr && (c.kdiag || c.rank < 1))) return false;
     const int64_t N = h.N, ld = lr ? c.rank + (c.rank & 1) : N;
     if (lr && ld > 2 * kRThreads) return false;
-    // one 256-thread block holds the whole state: the stage kernels' single-block sums
-    if (!lr && N <= 256) return false;
+    // one 256-thread block holds the whole state: the stage kernels' single-block sums; the
+    // timeout hook is for the low-rank and channel-wise kernels, dense runs complete with it
+    if (!lr && (N <= 256 || test_timeout)) return false;
     int dev = 0, nsm = 0, smem_max = 0, coop = 0;
     TDAGW_CUDA(cudaGetDevice(&dev));
     TDAGW_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));

@@ -59,3 +59,9 @@ def test_lowrank(L, nc, rank):
     U, S, V, d = wl.random_factors(p.N, rank, seed=rank + L)
     _run(p, tg.LOWRANK, lambda m: (lambda v: olr.apply_lowrank(d, U, S, V, v)),
          lambda c: tg.tdagw_set_factors(c.h, U, S, V, d))
+
+
+def test_dense_completes_with_the_timeout_hook():
+    ctx = tg.Context(wl.small_model(12, 1), tg.C64, stream=torch.cuda.current_stream().cuda_stream)
+    got = ctx.propagate(PULSE, 6, 0.2, tg.FULL, tg.FLAG_RESET | tg.FLAG_TEST_TIMEOUT)
+    np.testing.assert_array_equal(got, ctx.propagate(PULSE, 6, 0.2, tg.FULL, tg.FLAG_RESET | tg.FLAG_STAGEWISE))
