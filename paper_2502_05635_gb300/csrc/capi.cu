@@ -233,7 +233,7 @@ template <typename R> void get_factors(Ctx& c, double* U, double* S, double* V, 
 template <typename R> void apply(Ctx& c, int mode, const void* x, void* y, cudaStream_t s) {
     const int64_t N = c.hm.N;
     if (mode == TDAGW_FULL) {
-        launch_gemv<R>(c.K.p, N, N, N, x, y, 1, nullptr, nullptr, s);
+        launch_gemv<R>(c.K.p, N, N, N, x, y, s);
     } else if (mode == TDAGW_CHANNEL) {
         launch_ch_apply<R>(c, x, y, s);
     } else {

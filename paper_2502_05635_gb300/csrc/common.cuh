@@ -270,11 +270,10 @@ void launch_build_kernel(const Ctx& c, cudaStream_t s);
 template <typename R>
 void launch_gather_entries(const Ctx& c, const int64_t* rows, const int64_t* cols, int64_t n,
                            double2* out, cudaStream_t s);
-// y[row] (+ diag[row] * xd[row]) = sum_j A[row, j] x[j] for rows [0, nrows); with nsplit > 1
-// the columns are split and out holds nsplit partial vectors (no diag term then).
+// y[row] = sum_j A[row, j] x[j] for rows [0, nrows)
 template <typename R>
 void launch_gemv(const void* A, int64_t lda, int64_t nrows, int64_t ncols, const void* x,
-                 void* out, int nsplit, const void* diag, const void* xd, cudaStream_t s);
+                 void* out, cudaStream_t s);
 // part[b][c] = sum over row block b of conj(V[i][c]) x_i, V stored N x ldv (rows)
 template <typename R>
 void launch_vcols(const void* V, int64_t ldv, int64_t N, int r, const void* x, void* part,

@@ -49,24 +49,15 @@ __device__ __forceinline__ void ld2_cached(const double2* p, double2& a, double2
 
 // ---------------------------------------------------------------- GEMV ---------------
 
-// out[row] = sum_c A[row, c] x[c] (+ diag[row] xd[row]) for ROWS rows per block.  Each
-// thread walks the block's column range two complex at a time (16 B per row per step for
-// c64) so that a warp covers 512 contiguous bytes of each row per load; the ROWS
-// accumulators share every load of x.  nsplit > 1 splits the columns into nsplit ranges
-// and writes nsplit partial vectors (split-K) instead.
+// out[row] = sum_c A[row, c] x[c] for ROWS rows per block.  Each thread walks the columns two
+// complex at a time (16 B per row per step for c64) so that a warp covers 512 contiguous
+// bytes of each row per load; the ROWS accumulators share every load of x.
 template <typename R, int ROWS, int THREADS>
 __global__ void __launch_bounds__(THREADS)
 gemv_kernel(const cplx_t<R>* __restrict__ A, int64_t lda, int64_t nrows, int64_t ncols,
-            const cplx_t<R>* __restrict__ x, cplx_t<R>* __restrict__ out, int nsplit,
-            const cplx_t<R>* __restrict__ diag, const cplx_t<R>* __restrict__ xd) {
+            const cplx_t<R>* __restrict__ x, cplx_t<R>* __restrict__ out) {
     using C = cplx_t<R>;
-    const int64_t rg = blockIdx.x / nsplit;
-    const int split = blockIdx.x % nsplit;
-    const int64_t r0 = rg * ROWS;
-    int64_t cs = (ncols + nsplit - 1) / nsplit;
-    cs += cs & 1;
-    const int64_t c0 = split * cs;
-    const int64_t c1 = min(ncols, c0 + cs);
+    const int64_t r0 = (int64_t)blockIdx.x * ROWS;
     C acc[ROWS];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) acc[r] = mk((R)0, (R)0);
@@ -75,9 +66,9 @@ gemv_kernel(const cplx_t<R>* __restrict__ A, int64_t lda, int64_t nrows, int64_t
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) valid[r] = (r0 + r) < nrows;
 
-    int64_t c = c0 + 2 * tid;
+    int64_t c = 2 * tid;
 #pragma unroll 2
-    for (; c + 1 < c1; c += 2 * THREADS) {
+    for (; c + 1 < ncols; c += 2 * THREADS) {
         C x0, x1;
         ld2_cached(x + c, x0, x1);
         C a0[ROWS], a1[ROWS];
@@ -89,8 +80,8 @@ gemv_kernel(const cplx_t<R>* __restrict__ A, int64_t lda, int64_t nrows, int64_t
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) acc[r] = cfma(a1[r], x1, cfma(a0[r], x0, acc[r]));
     }
-    if (c1 > c0 && ((c1 - c0) & 1) && tid == 0) {
-        const int64_t cl = c1 - 1;
+    if ((ncols & 1) && tid == 0) {
+        const int64_t cl = ncols - 1;
         const C xl = x[cl];
 #pragma unroll
         for (int r = 0; r < ROWS; ++r)
@@ -112,13 +103,7 @@ gemv_kernel(const cplx_t<R>* __restrict__ A, int64_t lda, int64_t nrows, int64_t
         C s = red[0][tid];
 #pragma unroll
         for (int w = 1; w < NW; ++w) s = cadd(s, red[w][tid]);
-        const int64_t row = r0 + tid;
-        if (nsplit == 1) {
-            if (diag) s = cfma(diag[row], xd[row], s);
-            out[row] = s;
-        } else {
-            out[(int64_t)split * nrows + row] = s;
-        }
+        out[r0 + tid] = s;
     }
 }
 
@@ -491,14 +476,11 @@ void launch_kblock_add(const void* B, const void* x, void* y, int Nk, int P, cud
 
 template <typename R>
 void launch_gemv(const void* A, int64_t lda, int64_t nrows, int64_t ncols, const void* x,
-                 void* out, int nsplit, const void* diag, const void* xd, cudaStream_t s) {
+                 void* out, cudaStream_t s) {
     using C = cplx_t<R>;
     constexpr int ROWS = 4, THREADS = 256;
-    const int64_t rgs = (nrows + ROWS - 1) / ROWS;
-    const int64_t blocks = rgs * nsplit;
-    gemv_kernel<R, ROWS, THREADS><<<(unsigned)blocks, THREADS, 0, s>>>(
-        static_cast<const C*>(A), lda, nrows, ncols, static_cast<const C*>(x),
-        static_cast<C*>(out), nsplit, static_cast<const C*>(diag), static_cast<const C*>(xd));
+    gemv_kernel<R, ROWS, THREADS><<<(unsigned)((nrows + ROWS - 1) / ROWS), THREADS, 0, s>>>(
+        static_cast<const C*>(A), lda, nrows, ncols, static_cast<const C*>(x), static_cast<C*>(out));
     check_launch("gemv_kernel");
 }
 
@@ -606,8 +588,7 @@ void launch_observables_row(Ctx& c, const void* X, int64_t row, cudaStream_t s) 
 }
 
 #define INST(R)                                                                            \
-    template void launch_gemv<R>(const void*, int64_t, int64_t, int64_t, const void*, void*, \
-                                 int, const void*, const void*, cudaStream_t);             \
+    template void launch_gemv<R>(const void*, int64_t, int64_t, int64_t, const void*, void*, cudaStream_t); \
     template void launch_yreduce<R>(const void*, int, int, const void*, void*, cudaStream_t); \
     template void launch_vcols<R>(const void*, int64_t, int64_t, int, const void*, void*, int, \
                                   cudaStream_t);                                          \
