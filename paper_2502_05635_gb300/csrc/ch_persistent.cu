@@ -18,8 +18,8 @@
 // channels need all of x_p: every CTA publishes its rows of the stage input by pair after
 // the first barrier (when no CTA still reads the previous stage's), and reads x_p after
 // the second.  A producer warp streams the CTA's V rows and its U share through a
-// shared-memory ring with 1D bulk copies (L2 evict-first: the factors are read once per
-// stage), sixteen consumer warps compute from shared memory.
+// shared-memory ring with 1D bulk copies (L2 evict-first but for a share of U that stays in
+// L2: the factors are read once per stage), sixteen consumer warps compute from shared memory.
 // Every wait is bounded; on expiry the CTA records an error word and returns.
 #include <algorithm>
 
@@ -73,6 +73,7 @@ struct CHArgs {
     int* err;
     int T, nslots, slot_bytes, kmax, zs_len, upart_len;
     int vgroups;  // V pass: warp groups (power of two), each owning every vgroups-th pair
+    float keep;   // share of the U segments that stays in L2 between stages, in (0, 1]
     int extra_arrivals;  // > 0 only for the timeout test: the barrier can never complete
     unsigned long long wait_ns;
 };
@@ -168,12 +169,12 @@ __global__ void __launch_bounds__(kThr, 1) ch_persistent_kernel(CHArgs a) {
             RingPos pos{0, 0u};
             uint64_t issued = 0;
             bool ok = true;
-            const uint64_t policy = policy_evict_first();
             for (int n = 0; n < a.T && ok; ++n)
                 for (int st = 0; st < 4 && ok; ++st) {
                     // V pass: chunks of consecutive input pairs packed into shared slots
                     VWalk vw{0, 0, 0};
                     vw.skip_empty(a.m, P);
+                    const uint64_t vpolicy = policy_evict_first();
                     while (vw.q < P) {
                         if (issued >= (uint64_t)ns &&
                             !mbar_wait(empty + pos.slot, pos.phase ^ 1u, abort_s, a.wait_ns)) {
@@ -197,14 +198,20 @@ __global__ void __launch_bounds__(kThr, 1) ch_persistent_kernel(CHArgs a) {
                             const int ld = a.m.ldv[vw.q];
                             bulk_g2s_hint(ring + (size_t)pos.slot * a.slot_bytes + off,
                                           a.V + a.m.vbase[vw.q] + (int64_t)(ka + vw.r0) * ld, b, full + pos.slot,
-                                          policy);
+                                          vpolicy);
                             off += b;
                             vw.next(a.m, P, nk, nr);
                         }
                         ++issued;
                         pos.advance(1, ns);
                     }
-                    // U pass: this CTA's share, one chunk of rows of one pair per slot
+                    // U pass: this CTA's share, one chunk of rows of one pair per slot; a fixed
+                    // share of the lines (chosen by address) with normal priority, which
+                    // therefore stay in L2 from stage to stage, the others evict-first like V
+                    uint64_t policy;
+                    asm volatile("createpolicy.fractional.L2::evict_normal.L2::evict_first.b64 %0, %1;"
+                                 : "=l"(policy)
+                                 : "f"(a.keep));
                     for (int e = pA; e <= pB && ok; ++e) {
                         const int ld = a.m.ldw[e];
                         const int k0 = e == pA ? ur0 - pA * Nk : 0, k1 = e == pB ? ur1 - pB * Nk : Nk;
@@ -637,6 +644,13 @@ bool launch_ch_persistent(Ctx& c, int T, double dt, double dirx, double diry, bo
     // V-pass groups: as many as keep four columns per thread covering the longest V row
     a.vgroups = 1;
     while (a.vgroups < kCW && 4 * (kCons / (2 * a.vgroups)) >= maxv) a.vgroups *= 2;
+    // a quarter of L2 (32 MB) worth of U: with the V segments, x and the vectors it survives a
+    // stage's stream.  us / stage with 0, 15, 25, 40 MB: N = 20736 rank 65 (280 MB of factors)
+    // 53.8, 52.1, 50.4, 49.7; rank 130 (345 MB) 85.2, 85.2, 85.3, 85.9; N = 5184 rank 65 22.3, 21.8,
+    // 21.3, 20.9; N = 36864 rank 115 364.6 at each.  V kept instead of U: 54.0
+    int l2 = 0;
+    TDAGW_CUDA(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
+    a.keep = (float)std::min(1.0, 0.25 * (double)std::max(l2, 1) / (8.0 * (double)std::max<long long>(a.m.utot, 1)));
     a.extra_arrivals = test_timeout ? 1 : 0;
     a.wait_ns = test_timeout ? 20000000ull : 2000000000ull;
     void* args[] = {&a};
