@@ -52,8 +52,8 @@ __device__ __forceinline__ void ld2_cached(const double2* p, double2& a, double2
 // out[row] = sum_c A[row, c] x[c] for ROWS rows per block.  Each thread walks the columns two
 // complex at a time (16 B per row per step for c64) so that a warp covers 512 contiguous
 // bytes of each row per load; the ROWS accumulators share every load of x.  Bound by HBM:
-// 0.487 ms = 7.06 TB/s at N = 20736 in complex64 (0.541 with a split of the columns that no
-// call used any more: its bounds cost the loads their unrolled order).
+// 0.487 ms = 7.06 TB/s at N = 20736 in complex64 (0.541 while the kernel also had a split of
+// the columns, which no call used).
 template <typename R, int ROWS, int THREADS>
 __global__ void __launch_bounds__(THREADS)
 gemv_kernel(const cplx_t<R>* __restrict__ A, int64_t lda, int64_t nrows, int64_t ncols,
