@@ -1089,14 +1089,20 @@ __global__ void __launch_bounds__(kTcThreads, 1) batched_tc_kernel(TcArgs a) {
                 // every dSigma row is written before the epilogue reads it
                 if (in_sync && !(ok = tc_grid_sync(a, gen, &abort_s))) break;
                 TC_TRACE(worker && wt == 0, 7);
-                // ---- E (channel-wise): commutator + RK4 of all (k, trajectory) blocks, group by
-                //      group of trajectories, k-points dealt over the CTAs; a thread keeps one
-                //      trajectory and reads dSigma where phase C wrote it (staging it through
+                // ---- E (channel-wise): commutator + RK4 of all (k, trajectory) blocks; the CTAs
+                //      are dealt over the trajectory groups and share a group's k-points (578
+                //      -> 666 k traj-steps/s at N = 2304, B = 256 against every CTA in turn on
+                //      every group, one round of k-points each); a thread keeps one trajectory
+                //      and reads dSigma where phase C wrote it (staging it through
                 //      shared memory by 64-row tiles took two CTA barriers per tile and three
                 //      rounds of tiles on some CTAs: 18.5 -> 16.3 ms for 30 steps at N = 20736,
                 //      B = 64) ----
                 if (worker) {
-                    for (int g = 0; g < q.GC; ++g) {
+                    const int gs = min(q.GC, (int)gridDim.x), g0 = blockIdx.x % gs, slot = blockIdx.x / gs;
+                    const int nslots = ((int)gridDim.x - g0 + gs - 1) / gs;
+                    if (st == 3 && gs > 1)  // this CTA's partial sums of the other groups
+                        for (int e = wt; e < 3 * Bact; e += kWorkers) a.red[(int64_t)blockIdx.x * a.Bp * 3 + e] = 0.0;
+                    for (int g = g0; g < q.GC; g += gs) {
                         int b0, b1;
                         group_range(Bact, q.GC, g, b0, b1);
                         const int nbg = b1 - b0;
@@ -1111,7 +1117,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) batched_tc_kernel(TcArgs a) {
                             const int b = b0 + bl;
                             const float E = (float)a.Etab[(int64_t)b * a.ldE + 2 * (a.n0 + n) + eoff];
                             const float2 dr = a.dir[b];
-                            for (int k = blockIdx.x * kgroups + kg; k < a.Nk; k += gridDim.x * kgroups)
+                            for (int k = slot * kgroups + kg; k < a.Nk; k += nslots * kgroups)
                                 stage_kb_tc<NB, true>(a, k, b, st, E, dr, nullptr, 0, bl, xm, obs, -1);
                             atomicMax(smx + bl, __float_as_uint(xm));
                             if (st == 3) {
