@@ -15,12 +15,11 @@
 #include <vector>
 
 #include "common.cuh"
+#include "hhg_plan.h"
 
 namespace tdagw {
 
 namespace {
-
-constexpr int kHhgThreads = 128, kHhgChunk = 256;
 
 // part[(z nfreq + f) B + b]: the sum over the samples of block z's cpb chunks; with one block
 // along z the spectrum itself goes to out
@@ -43,7 +42,7 @@ hhg_kernel(const double* __restrict__ J, int64_t stride, int B, const int* __res
     for (int u = 0; u < TB; ++u) re[u] = im[u] = 0.0;
     for (int c = 0; c < cpb; ++c) {
         const int64_t n0 = ((int64_t)blockIdx.z * cpb + c) * clen;
-        const int cnt = (int)min((int64_t)clen, tmax + 1 - n0);
+        const int cnt = (int)min((int64_t)clen, (int64_t)tmax + 1 - n0);
         if (cnt <= 0) break;
         __syncthreads();
         for (int e = threadIdx.x; e < cnt * TB; e += kHhgThreads) {
@@ -99,19 +98,11 @@ void hhg_spectrum(const double* J, int64_t rows, int64_t stride, int B, const in
     int tmax = 0;
     for (int b = 0; b < B; ++b) tmax = std::max(tmax, steps[b]);
     TDAGW_REQUIRE(rows >= (int64_t)tmax + 1, TDAGW_ERR_INVALID_ARG, "fewer rows than steps + 1");
-    // the rows used (the last element read is ((tmax B + B - 1) stride)
-    const size_t nJ = ((size_t)(tmax + 1) * B - 1) * stride + 1;
-    // trajectories per thread, and chunks short enough to fill the GPU (a short run of a few
-    // trajectories is bound by the length of one thread's chain, not by the pipes)
-    const int TB = B >= 8 ? 8 : (B >= 4 ? 4 : 1);
+    // the rows used (the last element read is (tmax B + B - 1) stride)
+    const size_t nJ = (((size_t)tmax + 1) * B - 1) * stride + 1;
+    const HhgPlan pl = hhg_plan(tmax, B, nfreq);
     const int64_t per = (int64_t)nfreq * B;
-    const int64_t blocks = (int64_t)((nfreq + kHhgThreads - 1) / kHhgThreads) * ((B + TB - 1) / TB);
-    int clen = kHhgChunk;
-    while (clen > 32 && blocks * (tmax / clen + 1) < 2 * 152) clen /= 2;
-    // blocks along time: one per chunk while the partial sums stay below 64 MB
-    const int nchunk = tmax / clen + 1;
-    const int want = (int)std::max<int64_t>(1, std::min<int64_t>(nchunk, (int64_t)(1 << 22) / per));
-    const int cpb = (nchunk + want - 1) / want, nz = (nchunk + cpb - 1) / cpb;
+    const int nz = pl.nz;
     // one allocation: the partial sums, the result, omega, J, the step counts
     const size_t nO = (size_t)per, nP = nz > 1 ? 2 * nO * nz : 0;
     DevBuf buf;
@@ -122,10 +113,9 @@ void hhg_spectrum(const double* J, int64_t rows, int64_t stride, int B, const in
     TDAGW_CUDA(cudaMemcpyAsync(dJ, J, nJ * sizeof(double), cudaMemcpyHostToDevice, s));
     TDAGW_CUDA(cudaMemcpyAsync(dS, steps, (size_t)B * sizeof(int), cudaMemcpyHostToDevice, s));
     TDAGW_CUDA(cudaMemcpyAsync(dW, omega, (size_t)nfreq * sizeof(double), cudaMemcpyHostToDevice, s));
-    const dim3 grid((unsigned)((nfreq + kHhgThreads - 1) / kHhgThreads), (unsigned)((B + TB - 1) / TB),
-                    (unsigned)nz);
-    auto kern = TB == 8 ? hhg_kernel<8> : (TB == 4 ? hhg_kernel<4> : hhg_kernel<1>);
-    kern<<<grid, kHhgThreads, 0, s>>>(dJ, stride, B, dS, dt, dW, nfreq, clen, cpb, dP, dO);
+    const dim3 grid((unsigned)pl.gx, (unsigned)pl.gy, (unsigned)nz);
+    auto kern = pl.tb == 8 ? hhg_kernel<8> : (pl.tb == 4 ? hhg_kernel<4> : hhg_kernel<1>);
+    kern<<<grid, kHhgThreads, 0, s>>>(dJ, stride, B, dS, dt, dW, nfreq, pl.clen, pl.cpb, dP, dO);
     check_launch("hhg_kernel");
     if (nz > 1) {
         hhg_power_kernel<<<(unsigned)((per + kHhgThreads - 1) / kHhgThreads), kHhgThreads, 0, s>>>(dP, nz, dt, dW, nfreq,
