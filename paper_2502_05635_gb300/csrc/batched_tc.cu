@@ -301,18 +301,24 @@ __device__ void stage_kb_tc(const TcArgs& a, int k, int b, int st, float E, floa
     constexpr int NB2 = NB * NB;
     const int64_t Bp = a.Bp;
     float2 X[NB2], M[NB2];
+    if (GDS) {
+        // all rows of a partial before the next one: row after row, with a loop over a count
+        // known at run time in each, every load waits for the one before (N = 6400, 33
+        // trajectories, 10 steps: 2.41 -> 2.00 ms; N = 2304, 64 trajectories: 1.94 -> 1.85)
+#pragma unroll
+        for (int g = 0; g < NB2; ++g) M[g] = __ldcg(a.dS + ((int64_t)k * NB2 + g) * Bp + b);
+        for (int kc = 1; kc < a.kcu; ++kc) {
+#pragma unroll
+            for (int g = 0; g < NB2; ++g)
+                M[g] = cadd(M[g], __ldcg(a.dS + ((int64_t)kc * a.N + (int64_t)k * NB2 + g) * Bp + b));
+        }
+    }
 #pragma unroll
     for (int g = 0; g < NB2; ++g) {
         const int64_t i = (int64_t)k * NB2 + g;
         X[g] = __ldcg(a.X + i * Bp + b);
         const float2 d1 = a.dx[i], d2 = a.dy[i];
-        float2 ds;
-        if (GDS) {
-            ds = __ldcg(a.dS + i * Bp + b);
-            for (int kc = 1; kc < a.kcu; ++kc) ds = cadd(ds, __ldcg(a.dS + ((int64_t)kc * a.N + i) * Bp + b));
-        } else {
-            ds = cfma(a.diag[i], X[g], sDS[ds_index(row0 + g, bl)]);
-        }
+        const float2 ds = GDS ? M[g] : cfma(a.diag[i], X[g], sDS[ds_index(row0 + g, bl)]);
         if (rec >= 0) {  // stage input and dSigma, for the adjoint's backward sweep
             a.recX[rec + i * Bp + b] = X[g];
             a.recDS[rec + i * Bp + b] = ds;
@@ -1109,7 +1115,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) batched_tc_kernel(TcArgs a) {
                         workers_sync();  // the previous group's readers of smx and sred are done
                         if (wt < kGroup) smx[wt] = 0u;
                         workers_sync();
-                        const int kgroups = kWorkers / nbg;
+                        // no more k-points at a time than the group's CTAs need to share all of
+                        // them: a few trajectories would fill a few CTAs with one k-point per
+                        // thread and leave the others idle (N = 6400, one trajectory, 10 steps:
+                        // 3.05 ms with all that fit, 1.73 so; eight trajectories 1.81 and 1.76)
+                        const int kgroups = min(kWorkers / nbg, (a.Nk + nslots - 1) / nslots);
                         const int bl = wt % nbg, kg = wt / nbg;
                         DF3 obs;
                         float xm = 0.f;
@@ -1128,7 +1138,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) batched_tc_kernel(TcArgs a) {
                         }
                         workers_sync();
                         if (wt < nbg && !*vabort) {
-                            atomicMax(xout + b0 + wt, smx[wt]);
+                            if (slot * kgroups < a.Nk) atomicMax(xout + b0 + wt, smx[wt]);
                             if (st == 3) {
                                 double r0s = 0.0, r1s = 0.0, r2s = 0.0;
                                 for (int k2 = 0; k2 < kgroups; ++k2) {

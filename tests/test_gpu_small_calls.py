@@ -1,0 +1,64 @@
+"""Small calls on kernels whose work split is made for large ones: results against the FP64
+oracle where few trajectories or columns leave most threads without work, and that a call is not
+slower than one that has many times its work (best of several passes)."""
+import time
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_2502_05635_gb300 as tg  # noqa: E402
+import test_gpu_channel_tc as ctc  # noqa: E402
+import workloads as wl  # noqa: E402
+
+
+def _best(f, n=15):
+    for _ in range(3):
+        f()
+    torch.cuda.synchronize()
+    best = 1e30
+    for _ in range(n):
+        t0 = time.perf_counter()
+        f()
+        torch.cuda.synchronize()
+        best = min(best, time.perf_counter() - t0)
+    return best
+
+
+def _gauss(rng, *shape):
+    return (rng.standard_normal(shape) + 1j * rng.standard_normal(shape)) / np.sqrt(2 * shape[-2])
+
+
+@pytest.mark.parametrize("L,nc,B", [(12, 1, 1), (13, 1, 2), (5, 2, 3), (9, 2, 5), (9, 2, 1)])
+def test_split_channel_few_trajectories_vs_oracle(L, nc, B):
+    """k-points fewer, as many and more than the CTAs, one to five trajectories of uneven
+    lengths; the bar of the split-FP16 paths (1e-4)."""
+    p = wl.small_model(L, nc)
+    mdl, fac, _ = ctc._factors(p, 5)
+    c = ctc._ctx(p)
+    tg.tdagw_set_channel_factors(c.h, fac[1], fac[2], fac[3], fac[0])
+    pulses, steps = ctc._pulses(B, 7 * L + B), [40 - 7 * b for b in range(B)]
+    got = c.propagate_batch(pulses, steps, 0.2, tg.CHANNEL, ctc.SPLIT).reshape(41, B, 3)
+    c.close()
+    ctc._check_vs_oracle(mdl, fac, got, pulses, steps)
+
+
+def test_split_channel_one_trajectory_not_slower_than_64():
+    p = wl.small_model(20, 2)
+    P, Nk, z = p.Nb ** 2, 400, 4
+    rng = np.random.default_rng(3)
+    U = _gauss(rng, P, P, Nk, z)
+    S = 1e-2 * np.exp(-4.0 * np.arange(z) / z) * np.ones((P, P, 1))
+    c = ctc._ctx(p)
+    tg.tdagw_set_channel_factors(c.h, U, S, U)
+    pulses = ctc._pulses(64, 1)
+    one = _best(lambda: c.propagate_batch(pulses[:1], [40], 0.2, tg.CHANNEL, ctc.SPLIT))
+    many = _best(lambda: c.propagate_batch(pulses, [40] * 64, 0.2, tg.CHANNEL, ctc.SPLIT))
+    c.close()
+    print(f"one {one * 1e3:.3f} ms, 64 {many * 1e3:.3f} ms")
+    assert one < many, (one, many)
