@@ -186,8 +186,11 @@ __global__ void __launch_bounds__(kThreads, 1) lr_persistent_kernel(LRArgs a) {
         // ------------------------------------------------------------ consumer warps
         const int64_t ea = ra, eb = rb;
         const int jr0 = (int)((int64_t)cta * a.r / G), jr1 = (int)((int64_t)(cta + 1) * a.r / G);
-        // V pass by row subsets: vsub of them (1: all rows, more than 256 column pairs)
-        const int vsub = ldu <= kConsumers ? 2 * kConsumers / ldu : 1;
+        // V pass by row subsets: vsub of them (1: all rows, more than 256 column pairs), no more
+        // than a tile has rows: the subsets' sums are added one after the other, and at rank 1
+        // 512 of them, nearly all empty, cost more than the pass (N = 2116 with k-block
+        // diagonals: 10.4 -> 7.4 us / stage)
+        const int vsub = ldu <= kConsumers ? min(2 * kConsumers / ldu, min(rps, nrows)) : 1;
         const int vcp = vsub > 1 ? tid % (ldu / 2) : 0, vsb = vsub > 1 ? tid / (ldu / 2) : 0;
         unsigned lgen = 0;
         RingPos pos{0, 0u};

@@ -216,8 +216,10 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(ResArgs a) {
         const int n = gs >> 2, st = gs & 3, par = gs & 1;
         const float E = (float)__ldg(a.Etab + 2 * (int64_t)n + (st == 0 ? 0 : (st == 3 ? 2 : 1)));
         if (LR) {
-            // ---- V pass: thread = (column pair, subset of the rows)
-            const int ncp = ld / 2, nsub = kRThreads / ncp, cp = tid % ncp, sb = tid / ncp;
+            // ---- V pass: thread = (column pair, subset of the rows); no more subsets than rows
+            // (below, than CTAs): their sums are added one after the other, and a low rank would
+            // make up to 512 of them, nearly all empty (N = 2116, rank 1: 9.6 -> 4.4 us / stage)
+            const int ncp = ld / 2, nsub = min(kRThreads / ncp, nrows), cp = tid % ncp, sb = tid / ncp;
             float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
             if (sb < nsub) {
                 float2 y0 = zero, y1 = zero;
@@ -260,7 +262,7 @@ __global__ void __launch_bounds__(kRThreads, 1) resident_kernel(ResArgs a) {
         if (st == 0 && cta == G - 1 && warp == kRWarps - 1) write_observables(n);
         if (LR) {
             // ---- S o sum of all partial vectors: thread = (column pair, subset of the CTAs)
-            const int ncp = ld / 2, nsub = kRThreads / ncp, cp = tid % ncp, sb = tid / ncp;
+            const int ncp = ld / 2, nsub = min(kRThreads / ncp, G), cp = tid % ncp, sb = tid / ncp;
             float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
             const float4* src = reinterpret_cast<const float4*>((CL ? pcl : a.xch) + (int64_t)par * G * ld) + cp;
             if (sb < nsub) {

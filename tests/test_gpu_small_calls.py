@@ -62,3 +62,22 @@ def test_split_channel_one_trajectory_not_slower_than_64():
     c.close()
     print(f"one {one * 1e3:.3f} ms, 64 {many * 1e3:.3f} ms")
     assert one < many, (one, many)
+
+
+@pytest.mark.parametrize("L,nc,kblocks", [(12, 1, 0), (23, 1, 0), (36, 1, 0), (13, 2, 0), (23, 1, 1)],
+                         ids=["cluster", "grid", "large-grid", "nb4-grid", "streamed"])
+def test_lowest_ranks_not_slower_than_sixteen(L, nc, kblocks):
+    """One trajectory at ranks 1 and 2 (on-chip kernel; with k-block diagonals the streaming one):
+    the sums of the row subsets may not outgrow the products.  At rank 16 there are at most 64 of
+    them, at ranks 1 and 2 as many as a CTA has rows: half as much again is allowed."""
+    p = wl.small_model(L, nc)
+    P, t = p.Nb ** 2, {}
+    for rank in (1, 2, 16):
+        U, S, V, d = wl.random_factors(p.N, rank, seed=rank)
+        c = ctc._ctx(p)
+        tg.tdagw_set_kdiag_blocks(c.h, kblocks)
+        tg.tdagw_set_factors(c.h, U, S, V, np.zeros((L * L, P, P), complex) if kblocks else d)
+        t[rank] = _best(lambda: c.propagate(wl.Pulse(E0=1e-3), 100, 0.2, tg.LOWRANK))
+        c.close()
+    print({k: round(v * 1e6, 1) for k, v in t.items()})
+    assert max(t[1], t[2]) < 1.5 * t[16], t
