@@ -251,8 +251,12 @@ urows_kernel(const cplx_t<R>* __restrict__ A, int64_t lda, int64_t nrows, int nc
 constexpr int kClThreads = 512, kClCtas = 8, kClMaxRank = 512;
 // N r at most: N = 576, rank 29 takes 7.2 us a call (14.4 with three launches and the former
 // reductions), rank 110 10.3 (rank 120 with three launches 14.4); N = 2304, rank 28 12.3 (rank
-// 30 15.4).  Complex64 only: in complex128 eight SMs' FP64 pipes are slower than three launches.
-constexpr int64_t kClMaxElems = 65536;
+// 30 15.4).  And N at most: eight CTAs walk all rows, 256 a pass, so a low rank does not make a
+// large model cheap.  us per call of a series, one cluster against three launches, at ranks 3
+// and 12: N = 1296 10.3 and 14.4, 8.4 and 14.4; N = 2704 14.5 and 14.5, 12.4 and 16.5; N = 3600 16.6
+// and 15.5, 15.5 and 16.5; N = 5184 22.4 and 15.5, 20.5 and 16.5; N = 20736 rank 3 67.7 and 23.7.
+// Complex64 only: in complex128 eight SMs' FP64 pipes are slower than three launches.
+constexpr int64_t kClMaxElems = 65536, kClMaxN = 3072;
 template <typename R>
 __global__ void __cluster_dims__(kClCtas, 1, 1) __launch_bounds__(kClThreads)
 lr_cluster_kernel(const cplx_t<R>* __restrict__ U, const cplx_t<R>* __restrict__ V, int64_t ld, int N, int r,
@@ -525,7 +529,7 @@ template <typename R>
 void launch_lowrank_apply(const void* U, const void* V, int64_t ld, int64_t N, int r, const void* S, const void* diag,
                           const void* x, void* y, void* part, int nblocks, void* ytil, cudaStream_t s) {
     using C = cplx_t<R>;
-    if (sizeof(R) == 4 && r <= kClMaxRank && N * r <= kClMaxElems) {
+    if (sizeof(R) == 4 && r <= kClMaxRank && N <= kClMaxN && N * r <= kClMaxElems) {
         lr_cluster_kernel<R><<<kClCtas, kClThreads, 0, s>>>(
             static_cast<const C*>(U), static_cast<const C*>(V), ld, (int)N, r, static_cast<const R*>(S),
             static_cast<const C*>(diag), static_cast<const C*>(x), static_cast<C*>(y));

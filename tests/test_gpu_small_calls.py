@@ -81,3 +81,27 @@ def test_lowest_ranks_not_slower_than_sixteen(L, nc, kblocks):
         c.close()
     print({k: round(v * 1e6, 1) for k, v in t.items()})
     assert max(t[1], t[2]) < 1.5 * t[16], t
+
+
+def test_apply_of_a_low_rank_not_slower_than_of_four_times_the_rank():
+    """N = 20736: the rules by N r may not send a low rank of a large model to a kernel for small
+    models."""
+    p = wl.small_model(36, 2)
+    c, t = ctc._ctx(p), {}
+    x = torch.randn(p.N, dtype=torch.complex64, device="cuda")
+    y = torch.empty_like(x)
+    for rank in (3, 12):
+        U, S, V, d = wl.random_factors(p.N, rank, seed=rank)
+        tg.tdagw_set_factors(c.h, U, S, V, d)
+        t[rank] = _best(lambda: [tg.tdagw_apply(c.h, tg.LOWRANK, x, y) for _ in range(50)])
+    c.close()
+    print({k: round(v * 2e4, 1) for k, v in t.items()})
+    assert t[3] < 1.1 * t[12], t
+
+
+@pytest.mark.parametrize("L,nc,rank", [(13, 2, 24), (27, 1, 22), (28, 1, 20), (14, 2, 20)])
+def test_apply_on_both_sides_of_the_cluster_kernels_largest_model(L, nc, rank):
+    """N = 2704, 2916 | 3136, 3136 (the line is 3072), N rank within its bound on both sides; bound as
+    in the tests of the application's edges."""
+    import test_gpu_apply_edges as edges
+    edges.test_apply_lowrank_edges(L, nc, rank, tg.C64, 1e-6)
