@@ -320,7 +320,9 @@ lr_cluster_kernel(const cplx_t<R>* __restrict__ U, const cplx_t<R>* __restrict__
 // ---------------------------------------------------------------- stage --------------
 
 // Block partial sums of (P_x, J_x, occ_c1) in FP64, then the last block to arrive adds
-// the partials in block order (deterministic) and stores row `row` of obs.
+// the partials in a fixed order and stores row `row` of obs.  Up to 32 blocks one warp does it: the
+// full block's two levels of shuffles and its barriers cost more than one thread's sum did (dense,
+// N = 256, 100 steps: 2.40 ms with one thread, 2.49 with the block, 2.34 with one warp).
 __device__ void reduce_observables(double v0, double v1, double v2, double* red,
                                    unsigned* counter, double* obs_row, double inv_nk,
                                    int64_t* step_to_bump, int64_t new_step) {
@@ -353,11 +355,26 @@ __device__ void reduce_observables(double v0, double v1, double v2, double* red,
         last = (t == gridDim.x - 1);
     }
     __syncthreads();
-    if (last) {
-        // the last block's threads share the blocks' partials (fixed order); one thread alone
-        // waited for every one of them in turn
-        __threadfence();
-        double a = 0, b = 0, c = 0;
+    if (!last) return;
+    __threadfence();
+    double a = 0, b = 0, c = 0;
+    if (gridDim.x <= 32) {
+        // one warp, one partial per lane, as many halvings as there are partials
+        if (warp == 0) {
+            if (lane < (int)gridDim.x) {
+                a = __ldcg(red + lane * 3 + 0);
+                b = __ldcg(red + lane * 3 + 1);
+                c = __ldcg(red + lane * 3 + 2);
+            }
+            for (int o = 16; o > 0; o >>= 1)
+                if (o < (int)gridDim.x) {
+                    a += __shfl_xor_sync(0xffffffffu, a, o);
+                    b += __shfl_xor_sync(0xffffffffu, b, o);
+                    c += __shfl_xor_sync(0xffffffffu, c, o);
+                }
+        }
+    } else {
+        // the block's threads share the blocks' partials (fixed order)
         for (unsigned q = threadIdx.x; q < gridDim.x; q += blockDim.x) {
             a += __ldcg(red + q * 3 + 0);
             b += __ldcg(red + q * 3 + 1);
@@ -374,18 +391,19 @@ __device__ void reduce_observables(double v0, double v1, double v2, double* red,
             sred[warp][2] = c;
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == 0)
             for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
                 a += sred[w][0];
                 b += sred[w][1];
                 c += sred[w][2];
             }
-            obs_row[0] = a * inv_nk;
-            obs_row[1] = b * inv_nk;
-            obs_row[2] = c * inv_nk;
-            *counter = 0u;
-            if (step_to_bump) *step_to_bump = new_step;
-        }
+    }
+    if (threadIdx.x == 0) {
+        obs_row[0] = a * inv_nk;
+        obs_row[1] = b * inv_nk;
+        obs_row[2] = c * inv_nk;
+        *counter = 0u;
+        if (step_to_bump) *step_to_bump = new_step;
     }
 }
 
