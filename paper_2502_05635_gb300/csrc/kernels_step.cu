@@ -138,15 +138,18 @@ vcols_kernel(const cplx_t<R>* __restrict__ V, int64_t ldv, int64_t N, int r,
 // per block (128 or 256 contiguous bytes), the partials split over the rest of the threads (four
 // loads in flight each) and combined in a fixed order: one thread per column took a chain of
 // up to 304 loads (about 50 us).  Narrow blocks in FP64, whose additions would otherwise queue
-// at the pipes of a few SMs.
+// at the pipes of a few SMs.  subs: threads per column; a few partials (small models) get as many
+// as they need and one barrier, not the halvings of a full block (N = 144, channel-wise stage by
+// stage, us per stage with one thread per column, a full block and this: 17.2, 17.9, 17.2 in complex64,
+// 21.9, 22.8, 20.2 in complex128).
 constexpr int kYThreads = 512;
 template <typename R> constexpr int kYCols = sizeof(R) == 8 ? 8 : 32;
-template <typename R>
-__global__ void __launch_bounds__(kYThreads)
+template <typename R, int subs>
+__global__ void __launch_bounds__(subs * kYCols<R>)
 yreduce_kernel(const cplx_t<R>* __restrict__ part, int nsplit, int r, const R* __restrict__ S,
                cplx_t<R>* __restrict__ ytil) {
     using C = cplx_t<R>;
-    constexpr int cols = kYCols<R>, subs = kYThreads / cols;
+    constexpr int cols = kYCols<R>;
     const int col = threadIdx.x % cols, sub = threadIdx.x / cols;
     const int j = blockIdx.x * cols + col;
     const int q0 = (int)((int64_t)sub * nsplit / subs), q1 = (int)((int64_t)(sub + 1) * nsplit / subs);
@@ -160,15 +163,31 @@ yreduce_kernel(const cplx_t<R>* __restrict__ part, int nsplit, int r, const R* _
 #pragma unroll
             for (int u = 0; u < 4; ++u) s[u] = cadd(s[u], part[(int64_t)(q + u) * r + j]);
         }
-        for (; q < q1; ++q) s[0] = cadd(s[0], part[(int64_t)q * r + j]);
-    }
-    red[sub][col] = cadd(cadd(s[0], s[1]), cadd(s[2], s[3]));
+        if (subs <= 4) {
 #pragma unroll
-    for (int o = subs / 2; o > 0; o >>= 1) {
-        __syncthreads();
-        if (sub < o) red[sub][col] = cadd(red[sub][col], red[sub + o][col]);
+            for (int u = 0; u < 3; ++u)
+                if (q + u < q1) s[u] = cadd(s[u], part[(int64_t)(q + u) * r + j]);
+        } else {
+            for (; q < q1; ++q) s[0] = cadd(s[0], part[(int64_t)q * r + j]);
+        }
     }
-    if (sub == 0 && j < r) ytil[j] = cscale(red[0][col], S[j]);
+    C t = cadd(cadd(s[0], s[1]), cadd(s[2], s[3]));
+    red[sub][col] = t;
+    if (subs <= 4) {
+        __syncthreads();
+        if (sub == 0) {
+#pragma unroll
+            for (int u = 1; u < subs; ++u) t = cadd(t, red[u][col]);
+        }
+    } else {
+#pragma unroll
+        for (int o = subs / 2; o > 0; o >>= 1) {
+            __syncthreads();
+            if (sub < o) red[sub][col] = cadd(red[sub][col], red[sub + o][col]);
+        }
+        t = red[sub][col];
+    }
+    if (sub == 0 && j < r) ytil[j] = cscale(t, S[j]);
 }
 
 // Sums of W rows held one partial per lane: W 2^k halvings across the lanes, then plain
@@ -523,9 +542,11 @@ template <typename R>
 void launch_yreduce(const void* part, int nsplit, int r, const void* S, void* ytil,
                     cudaStream_t s) {
     using C = cplx_t<R>;
-    yreduce_kernel<R><<<(r + kYCols<R> - 1) / kYCols<R>, kYThreads, 0, s>>>(static_cast<const C*>(part), nsplit, r,
-                                                       static_cast<const R*>(S),
-                                                       static_cast<C*>(ytil));
+    constexpr int full = kYThreads / kYCols<R>;
+    const int subs = nsplit <= 4 ? 1 : (nsplit <= 16 ? 4 : full);
+    auto k = subs == 1 ? yreduce_kernel<R, 1> : (subs == 4 ? yreduce_kernel<R, 4> : yreduce_kernel<R, full>);
+    k<<<(r + kYCols<R> - 1) / kYCols<R>, subs * kYCols<R>, 0, s>>>(static_cast<const C*>(part), nsplit, r,
+                                                                 static_cast<const R*>(S), static_cast<C*>(ytil));
     check_launch("yreduce_kernel");
 }
 

@@ -1,7 +1,8 @@
-"""The stage-wise single-trajectory kernels at the edges of their sums: the last block's sum of the
-blocks' observables (one block, 31 to 34 of them, and more; 256 threads in complex64, 32 in
-complex128), against the FP64 oracle.  Tolerances: those of the propagation tests, 1e-5 and 1e-10
-relative L2 for the two precisions."""
+"""The stage-wise single-trajectory kernels at the edges of their sums, against the FP64 oracle: the
+last block's sum of the blocks' observables (one block, 31 to 34 of them, and more; 256 threads in
+complex64, 32 in complex128), and the sum of the V pass's partial vectors (one per 16 rows: 1, 3 to
+5, 15 to 17 and more).  Tolerances: those of the propagation tests, 1e-5 and 1e-10 relative L2 for
+the two precisions, and of the application tests, 2e-6 and 1e-12 of the largest entry."""
 import numpy as np
 import pytest
 
@@ -13,6 +14,7 @@ if not torch.cuda.is_available():  # pragma: no cover
 
 import paper_2502_05635_gb300 as tg  # noqa: E402
 import workloads as wl  # noqa: E402
+from oracle import channel as oc  # noqa: E402
 from oracle import lowrank as olr  # noqa: E402
 from oracle import model as om  # noqa: E402
 from oracle import propagate as op  # noqa: E402
@@ -40,3 +42,27 @@ def test_observables_over_block_counts(L, nc, dtype, tol):
     c.close()
     for j in range(3):
         assert op.rel_l2(got[1:, j], ref[1:, j]) < tol, j
+
+
+@pytest.mark.parametrize("dtype,tol", [(tg.C64, 2e-6), (tg.C128, 1e-12)], ids=["c64", "c128"])
+@pytest.mark.parametrize("L,nc", [(1, 1), (3, 1), (4, 1), (5, 1), (2, 2), (8, 1), (4, 2), (9, 1), (17, 1), (5, 2)])
+def test_partial_vector_counts(L, nc, dtype, tol):
+    p = wl.small_model(L, nc)
+    P, Nk, r = p.Nb ** 2, L * L, min(3, L * L)
+    rng = np.random.default_rng(L)
+    g = lambda *s: (rng.standard_normal(s) + 1j * rng.standard_normal(s)) / np.sqrt(2 * Nk)
+    U, V, D, S = g(P, P, Nk, r), g(P, P, Nk, r), g(P, Nk, Nk), rng.uniform(0.1, 1.0, (P, P, r))
+    for q in range(P):
+        U[q, q] = V[q, q] = 0
+        S[q, q] = 0
+    Ul, Sl, Vl, dl = wl.random_factors(p.N, min(5, p.N), seed=L)
+    c = _ctx(p, dtype)
+    tg.tdagw_set_channel_factors(c.h, U, S, V, D)
+    tg.tdagw_set_factors(c.h, Ul, Sl, Vl, dl)
+    x = wl.random_state(p.N, 3)
+    tx = torch.from_numpy(x).to("cuda", torch.complex64 if dtype == tg.C64 else torch.complex128)
+    for mode, ref in ((tg.CHANNEL, oc.apply_channel(D, U, S, V, x)), (tg.LOWRANK, olr.apply_lowrank(dl, Ul, Sl, Vl, x))):
+        y = torch.full_like(tx, float("nan"))
+        tg.tdagw_apply(c.h, mode, tx, y)
+        assert np.abs(y.cpu().numpy() - ref).max() < tol * np.abs(ref).max(), mode
+    c.close()
