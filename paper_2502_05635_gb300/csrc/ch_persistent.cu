@@ -73,7 +73,7 @@ struct CHArgs {
     int* err;
     int T, nslots, slot_bytes, kmax, zs_len, upart_len;
     int vgroups;  // V pass: warp groups (power of two), each owning every vgroups-th pair
-    float keep;   // share of the U segments that stays in L2 between stages, in (0, 1]
+    float keep;   // share of the U segments that stays in L2 between stages (0: all evict-first)
     int extra_arrivals;  // > 0 only for the timeout test: the barrier can never complete
     unsigned long long wait_ns;
 };
@@ -169,12 +169,19 @@ __global__ void __launch_bounds__(kThr, 1) ch_persistent_kernel(CHArgs a) {
             RingPos pos{0, 0u};
             uint64_t issued = 0;
             bool ok = true;
+            // U: a fixed share of the lines (chosen by address) with normal priority, which
+            // therefore stay in L2 from stage to stage, the others evict-first like V
+            const uint64_t vpolicy = policy_evict_first();
+            uint64_t policy = vpolicy;
+            if (a.keep > 0.f)
+                asm volatile("createpolicy.fractional.L2::evict_normal.L2::evict_first.b64 %0, %1;"
+                             : "=l"(policy)
+                             : "f"(a.keep));
             for (int n = 0; n < a.T && ok; ++n)
                 for (int st = 0; st < 4 && ok; ++st) {
                     // V pass: chunks of consecutive input pairs packed into shared slots
                     VWalk vw{0, 0, 0};
                     vw.skip_empty(a.m, P);
-                    const uint64_t vpolicy = policy_evict_first();
                     while (vw.q < P) {
                         if (issued >= (uint64_t)ns &&
                             !mbar_wait(empty + pos.slot, pos.phase ^ 1u, abort_s, a.wait_ns)) {
@@ -205,13 +212,7 @@ __global__ void __launch_bounds__(kThr, 1) ch_persistent_kernel(CHArgs a) {
                         ++issued;
                         pos.advance(1, ns);
                     }
-                    // U pass: this CTA's share, one chunk of rows of one pair per slot; a fixed
-                    // share of the lines (chosen by address) with normal priority, which
-                    // therefore stay in L2 from stage to stage, the others evict-first like V
-                    uint64_t policy;
-                    asm volatile("createpolicy.fractional.L2::evict_normal.L2::evict_first.b64 %0, %1;"
-                                 : "=l"(policy)
-                                 : "f"(a.keep));
+                    // U pass: this CTA's share, one chunk of rows of one pair per slot
                     for (int e = pA; e <= pB && ok; ++e) {
                         const int ld = a.m.ldw[e];
                         const int k0 = e == pA ? ur0 - pA * Nk : 0, k1 = e == pB ? ur1 - pB * Nk : Nk;
@@ -647,10 +648,14 @@ bool launch_ch_persistent(Ctx& c, int T, double dt, double dirx, double diry, bo
     // a quarter of L2 (32 MB) worth of U: with the V segments, x and the vectors it survives a
     // stage's stream.  us / stage with 0, 15, 25, 40 MB: N = 20736 rank 65 (280 MB of factors)
     // 53.8, 52.1, 50.4, 49.7; rank 130 (345 MB) 85.2, 85.2, 85.3, 85.9; N = 5184 rank 65 22.3, 21.8,
-    // 21.3, 20.9; N = 36864 rank 115 364.6 at each.  V kept instead of U: 54.0
+    // 21.3, 20.9; N = 36864 rank 115 364.6 at each.  V kept instead of U: 54.0.  Nothing kept of
+    // segments below an eighth of L2 (a sixteenth with four bands), which fit in any case: there
+    // it costs up to 1 % (us / stage without and with it: N = 484 rank 2 14.8, 14.9; N = 2500 rank
+    // 75 16.0, 16.1), above it gains (N = 3136 rank 39 17.0, 16.6; four bands, N = 5184 rank 16 23.4, 22.9)
     int l2 = 0;
     TDAGW_CUDA(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
-    a.keep = (float)std::min(1.0, 0.25 * (double)std::max(l2, 1) / (8.0 * (double)std::max<long long>(a.m.utot, 1)));
+    const double ubytes = 8.0 * (double)a.m.utot;
+    a.keep = ubytes > l2 / (h.Nb == 2 ? 8 : 16) ? (float)std::min(1.0, 0.25 * (double)l2 / ubytes) : 0.f;
     a.extra_arrivals = test_timeout ? 1 : 0;
     a.wait_ns = test_timeout ? 20000000ull : 2000000000ull;
     void* args[] = {&a};
