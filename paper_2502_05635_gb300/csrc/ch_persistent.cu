@@ -660,7 +660,8 @@ bool launch_ch_persistent(Ctx& c, int T, double dt, double dirx, double diry, bo
     a.wait_ns = test_timeout ? 20000000ull : 2000000000ull;
     void* args[] = {&a};
     const void* fn = h.Nb == 2 ? (const void*)ch_persistent_kernel<2> : (const void*)ch_persistent_kernel<4>;
-    TDAGW_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the same limit for every model: a launch by another thread must not find it lowered
+    TDAGW_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)avail));
     int per_sm = 0;
     TDAGW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThr, smem));
     if (per_sm < 1) return false;

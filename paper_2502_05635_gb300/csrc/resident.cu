@@ -392,7 +392,8 @@ bool launch_resident(Ctx& c, int mode, int T, double dt, double dirx, double dir
     if (cl) {
         const void* fn = kernel(true);
         const size_t sm = smem_for(rows_of(G), G);
-        TDAGW_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        // the same limit for every model: a launch by another thread must not find it lowered
+        TDAGW_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap));
         TDAGW_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         attr.id = cudaLaunchAttributeClusterDimension;
         attr.val.clusterDim.x = (unsigned)G;
@@ -463,7 +464,7 @@ bool launch_resident(Ctx& c, int mode, int T, double dt, double dirx, double dir
         TDAGW_CUDA(cudaLaunchKernelExC(&cfg, fn, args));
     } else {
         const size_t smem = smem_for(rows_max, 0);
-        TDAGW_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        TDAGW_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap));
         int per_sm = 0;
         TDAGW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kRThreads, smem));
         if (per_sm < 1) return false;
