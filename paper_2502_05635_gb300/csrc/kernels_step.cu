@@ -144,10 +144,10 @@ vcols_kernel(const cplx_t<R>* __restrict__ V, int64_t ldv, int64_t N, int r,
 // 21.9, 22.8, 20.2 in complex128).
 constexpr int kYThreads = 512;
 template <typename R> constexpr int kYCols = sizeof(R) == 8 ? 8 : 32;
+template <typename R> constexpr int kYSubs = kYThreads / kYCols<R>;
 template <typename R, int subs>
-__global__ void __launch_bounds__(subs * kYCols<R>)
-yreduce_kernel(const cplx_t<R>* __restrict__ part, int nsplit, int r, const R* __restrict__ S,
-               cplx_t<R>* __restrict__ ytil) {
+__device__ __forceinline__ void yreduce(const cplx_t<R>* __restrict__ part, int nsplit, int r, const R* __restrict__ S,
+                                        cplx_t<R>* __restrict__ ytil) {
     using C = cplx_t<R>;
     constexpr int cols = kYCols<R>;
     const int col = threadIdx.x % cols, sub = threadIdx.x / cols;
@@ -188,6 +188,18 @@ yreduce_kernel(const cplx_t<R>* __restrict__ part, int nsplit, int r, const R* _
         t = red[sub][col];
     }
     if (sub == 0 && j < r) ytil[j] = cscale(t, S[j]);
+}
+template <typename R>
+__global__ void __launch_bounds__(kYThreads)
+yreduce_kernel(const cplx_t<R>* __restrict__ part, int nsplit, int r, const R* __restrict__ S,
+               cplx_t<R>* __restrict__ ytil) {
+    yreduce<R, kYSubs<R>>(part, nsplit, r, S, ytil);
+}
+template <typename R, int subs>
+__global__ void __launch_bounds__(subs * kYCols<R>)
+yreduce_few_kernel(const cplx_t<R>* __restrict__ part, int nsplit, int r, const R* __restrict__ S,
+                   cplx_t<R>* __restrict__ ytil) {
+    yreduce<R, subs>(part, nsplit, r, S, ytil);
 }
 
 // Sums of W rows held one partial per lane: W 2^k halvings across the lanes, then plain
@@ -542,9 +554,8 @@ template <typename R>
 void launch_yreduce(const void* part, int nsplit, int r, const void* S, void* ytil,
                     cudaStream_t s) {
     using C = cplx_t<R>;
-    constexpr int full = kYThreads / kYCols<R>;
-    const int subs = nsplit <= 4 ? 1 : (nsplit <= 16 ? 4 : full);
-    auto k = subs == 1 ? yreduce_kernel<R, 1> : (subs == 4 ? yreduce_kernel<R, 4> : yreduce_kernel<R, full>);
+    const int subs = nsplit <= 4 ? 1 : (nsplit <= 16 ? 4 : kYSubs<R>);
+    auto k = subs == 1 ? yreduce_few_kernel<R, 1> : (subs == 4 ? yreduce_few_kernel<R, 4> : yreduce_kernel<R>);
     k<<<(r + kYCols<R> - 1) / kYCols<R>, subs * kYCols<R>, 0, s>>>(static_cast<const C*>(part), nsplit, r,
                                                                  static_cast<const R*>(S), static_cast<C*>(ytil));
     check_launch("yreduce_kernel");
