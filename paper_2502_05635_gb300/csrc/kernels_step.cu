@@ -288,12 +288,12 @@ constexpr int kClThreads = 512, kClCtas = 8, kClMaxRank = 512;
 // and 15.5, 15.5 and 16.5; N = 5184 22.4 and 15.5, 20.5 and 16.5; N = 20736 rank 3 67.7 and 23.7.
 // Complex64 only: in complex128 eight SMs' FP64 pipes are slower than three launches.
 constexpr int64_t kClMaxElems = 65536, kClMaxN = 3072;
-template <typename R>
 __global__ void __cluster_dims__(kClCtas, 1, 1) __launch_bounds__(kClThreads)
-lr_cluster_kernel(const cplx_t<R>* __restrict__ U, const cplx_t<R>* __restrict__ V, int64_t ld, int N, int r,
-                  const R* __restrict__ S, const cplx_t<R>* __restrict__ diag, const cplx_t<R>* __restrict__ x,
-                  cplx_t<R>* __restrict__ y) {
-    using C = cplx_t<R>;
+lr_cluster_kernel(const float2* __restrict__ U, const float2* __restrict__ V, int64_t ld, int N, int r,
+                  const float* __restrict__ S, const float2* __restrict__ diag, const float2* __restrict__ x,
+                  float2* __restrict__ y) {
+    using R = float;
+    using C = float2;
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     __shared__ __align__(16) C sub[2 * kClThreads];
@@ -579,12 +579,14 @@ template <typename R>
 void launch_lowrank_apply(const void* U, const void* V, int64_t ld, int64_t N, int r, const void* S, const void* diag,
                           const void* x, void* y, void* part, int nblocks, void* ytil, cudaStream_t s) {
     using C = cplx_t<R>;
-    if (sizeof(R) == 4 && r <= kClMaxRank && N <= kClMaxN && N * r <= kClMaxElems) {
-        lr_cluster_kernel<R><<<kClCtas, kClThreads, 0, s>>>(
-            static_cast<const C*>(U), static_cast<const C*>(V), ld, (int)N, r, static_cast<const R*>(S),
-            static_cast<const C*>(diag), static_cast<const C*>(x), static_cast<C*>(y));
-        check_launch("lr_cluster_kernel");
-        return;
+    if constexpr (sizeof(R) == 4) {
+        if (r <= kClMaxRank && N <= kClMaxN && N * r <= kClMaxElems) {
+            lr_cluster_kernel<<<kClCtas, kClThreads, 0, s>>>(
+                static_cast<const C*>(U), static_cast<const C*>(V), ld, (int)N, r, static_cast<const R*>(S),
+                static_cast<const C*>(diag), static_cast<const C*>(x), static_cast<C*>(y));
+            check_launch("lr_cluster_kernel");
+            return;
+        }
     }
     launch_vcols<R>(V, ld, N, r, x, part, nblocks, s);
     launch_yreduce<R>(part, nblocks, r, S, ytil, s);
