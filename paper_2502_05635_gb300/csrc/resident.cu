@@ -18,7 +18,9 @@
 // path of the dense kernel takes two launches per stage; the streaming low-rank kernel
 // (lr_persistent.cu) two barriers, and its state goes through L2.  The exchange buffers
 // alternate by stage parity: a CTA writes the next stage's while a slower one still reads.
-// Waits are bounded as in the other persistent kernels.
+// The grid form's waits are bounded as in the other persistent kernels (the timeout hook tests them
+// in its low-rank form).  The cluster form waits at the hardware's cluster barrier, which has no
+// budget: its CTAs are scheduled together, and none leaves before its last barrier.
 //
 // Measured per stage: dense, N = 576 6.1 us (stage-wise) -> 3.6 (grid) -> 2.7 (cluster); low
 // rank, N = 2116, rank 235 9.3 us (streaming kernel) -> 5.6 (grid).
@@ -358,8 +360,10 @@ bool launch_resident(Ctx& c, int mode, int T, double dt, double dirx, double dir
     if (c.dtype != TDAGW_C64 || (lr && (c.kdiag || c.rank < 1))) return false;
     const int64_t N = h.N, ld = lr ? c.rank + (c.rank & 1) : N;
     if (lr && ld > 2 * kRThreads) return false;
-    // one 256-thread block holds the whole state: the stage kernels' single-block sums; the
-    // timeout hook is for the low-rank and channel-wise kernels, dense runs complete with it
+    // up to 256 elements dense runs stay with the stage kernels: one block of theirs holds the whole
+    // state, and its FP64 sums of an undisturbed state give the exact zero that the tests hold at
+    // N = 256, where the double-float sums of several CTAs may leave 1e-17; the timeout hook is for
+    // the low-rank and channel-wise kernels, dense runs complete with it
     if (!lr && (N <= 256 || test_timeout)) return false;
     int dev = 0, nsm = 0, smem_max = 0, coop = 0;
     TDAGW_CUDA(cudaGetDevice(&dev));
@@ -413,12 +417,15 @@ bool launch_resident(Ctx& c, int mode, int T, double dt, double dirx, double dir
     }
     if (!cl) {
         // k-points per CTA: low rank about sqrt(N) CTAs (a CTA reads its share of the factors
-        // and one partial vector per CTA: 2 N / G + G rows, least at G = sqrt(N)); dense eight rows
+        // and one partial vector per CTA: 2 N / G + G rows, least at G = sqrt(N)), more where their
+        // shares do not fit; dense eight rows.  Whatever fits is taken: up to 152 partial vectors of
+        // 500 columns cost less than streaming the factors and a second barrier (us / stage streamed
+        // and on chip: N = 2116 rank 400 9.9 and 6.7, rank 500 10.4 and 8.6; N = 3600 rank 511 10.6 and 10.1; N = 5184
+        // rank 290 12.8 and 8.5; four bands, N = 4624 rank 400 12.2 and 9.0, N = 9216 rank 190 12.0 and 7.9)
         const int Gw = lr ? (int)std::lround(std::sqrt((double)N)) : (int)((N + 7) / 8);
         G = std::max(1, std::min({Gw, nsm, h.Nk}));
         while (G < std::min(nsm, h.Nk) && (rows_of(G) > kRThreads || smem_for(rows_of(G), 0) > cap)) ++G;
         if (rows_of(G) > kRThreads || smem_for(rows_of(G), 0) > cap) return false;
-        if (lr && (int64_t)G * ld * 8 > 160 * 1024) return false;
     }
     const int rows_max = rows_of(G);
 

@@ -1,4 +1,5 @@
-"""The forms of a single-trajectory call that a model's size no longer reaches by itself: runs
+"""On-chip low-rank runs with many columns over many CTAs, against the oracle and the stage-wise
+kernels, and the forms of a single-trajectory call that a model's size no longer reaches by itself: runs
 replayed from a captured graph against the same launches made directly (32 steps per replay, a
 tail of direct steps), continued runs on the stage-wise kernels, and the bounded waits of the
 streaming low-rank kernel beside those of the on-chip one."""
@@ -13,7 +14,9 @@ if not torch.cuda.is_available():  # pragma: no cover
 
 import paper_2502_05635_gb300 as tg  # noqa: E402
 import workloads as wl  # noqa: E402
+from oracle import lowrank as olr  # noqa: E402
 from oracle import propagate as op  # noqa: E402
+from test_gpu_resident import _run  # noqa: E402
 
 PULSE = wl.Pulse(E0=5e-3, omega=0.12, t0=3.0, sigma=1.2, dir_x=0.6, dir_y=0.8)
 
@@ -83,3 +86,13 @@ def test_lowrank_timeout_is_reported_and_context_survives(L, nc, rank, kblocks):
     ref = c.propagate(PULSE, 20, 0.2, tg.LOWRANK, tg.FLAG_RESET | tg.FLAG_STAGEWISE)
     assert op.rel_l2(good[:, 0], ref[:, 0]) < 1e-6
     c.close()
+
+
+@pytest.mark.parametrize("L,nc,rank", [(23, 1, 500), (30, 1, 511), (36, 1, 320), (17, 2, 400), (24, 2, 190)])
+def test_onchip_lowrank_with_long_exchange(L, nc, rank):
+    """Up to 152 partial vectors of up to 512 columns per stage; tolerances of the on-chip kernel's
+    other tests (the same sums)."""
+    p = wl.small_model(L, nc)
+    U, S, V, d = wl.random_factors(p.N, rank, seed=rank + L)
+    _run(p, tg.LOWRANK, lambda m: (lambda v: olr.apply_lowrank(d, U, S, V, v)),
+         lambda c: tg.tdagw_set_factors(c.h, U, S, V, d), T=12)
