@@ -419,8 +419,9 @@ static __device__ void kblock_term(const float2* __restrict__ kblk, const float2
     }
 }
 
-// The product with the tile that pads M least: the cost of a pass is that of its Mt rows
-// (512 threads x TM rows / slices), whatever the split.
+// The product with the tile of those built that pads M least: the cost of a pass is that of its Mt
+// rows (512 threads x TM rows / slices), whatever the split.  Heights 3 and 7 (17 to 24 and 49 to 56
+// rows) are not built; 4 and 8 take those.
 template <bool TRANS>
 static __device__ __forceinline__ void block_gemm(const float2* __restrict__ A, int64_t lda, int M, int Q,
                                   const float2* __restrict__ Bm, int64_t ldb, int nb,

@@ -281,7 +281,7 @@ void launch_vcols(const void* V, int64_t ldv, int64_t N, int r, const void* x, v
 template <typename R>
 void launch_yreduce(const void* part, int nsplit, int r, const void* S, void* ytil,
                     cudaStream_t s);
-// y = diag o x + U (S o (V^H x)) (diag nullptr: without): one cluster launch for small N r,
+// y = diag o x + U (S o (V^H x)) (diag nullptr: without): one cluster launch for small N and N r,
 // else the V pass into nblocks partial vectors (part, nblocks x r), their sum (ytil, r) and the
 // U pass.  U and V rows start on 16 bytes (even ld).
 template <typename R>
