@@ -1098,11 +1098,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) batched_tc_kernel(TcArgs a) {
                 // ---- E (channel-wise): commutator + RK4 of all (k, trajectory) blocks; the CTAs
                 //      are dealt over the trajectory groups and share a group's k-points (578
                 //      -> 666 k traj-steps/s at N = 2304, B = 256 against every CTA in turn on
-                //      every group, one round of k-points each); a thread keeps one trajectory
+                //      every group, one round of k-points each; 772 k with a partial's rows
+                //      loaded together); a thread keeps one trajectory
                 //      and reads dSigma where phase C wrote it (staging it through
                 //      shared memory by 64-row tiles took two CTA barriers per tile and three
-                //      rounds of tiles on some CTAs: 18.5 -> 16.3 ms for 30 steps at N = 20736,
-                //      B = 64) ----
+                //      rounds of tiles on some CTAs: 18.5 -> 17.3 ms for 30 steps at N = 20736,
+                //      B = 64; 16.7 with a partial's rows loaded together) ----
                 if (worker) {
                     const int gs = min(q.GC, (int)gridDim.x), g0 = blockIdx.x % gs, slot = blockIdx.x / gs;
                     const int nslots = ((int)gridDim.x - g0 + gs - 1) / gs;
