@@ -47,7 +47,7 @@ def test_two_sizes_from_four_threads(mode, sizes, kblocks):
             c = tg.Context(p, tg.C64, stream=st.cuda_stream)
             _factors(c, p, mode, rank, kblocks)
             first = c.propagate(PULSE, 2, 0.2, mode)
-            start.wait(30)
+            start.wait(120)
             f = [tg.make_field(PULSE)]
             for n in range(4000):  # launches follow one another: only every eighth result is read
                 tg.tdagw_propagate(c.h, f, [2], 0.2, mode)
